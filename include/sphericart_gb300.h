@@ -145,7 +145,8 @@ typedef enum {
  * DEGREE kernels read warps_per_block (0..8, 0 = by shared memory),
  * blocks_per_sm and lanes_per_point (1, 2 or 4 lanes per point for DEGREE, 0 =
  * by measurement; DEGREE_DOWN takes 1). ROW kernels read warps_per_block
- * (forward 0..2, backward 0..8; 0 = 1 forward, 2 with Hessians and backward),
+ * (forward 0..2, backward 0..8; 0 = one block of up to 12, backward 16, warps
+ * per SM, 2 with Hessians),
  * blocks_per_sm, and lanes_per_point as the forward window policy (0 = by
  * l_max, 1, 2; with Hessians 0/2 = 136 columns, 1 = one degree of l_max,
  * 3 = 256 columns).

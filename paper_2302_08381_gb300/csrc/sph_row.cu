@@ -72,37 +72,88 @@ struct CSf {
     }
 };
 
+// (x + i y)^e for 0 <= e < 8 from (x + i y)^1, ^2 and ^4: 9 complex products with
+// the squares where powers step by step took 30, of the ~1,000 operations a
+// tile's prologue and its degrees cost at l_max 20.
+__device__ __forceinline__ CSf row_power(const CSf& w1, const CSf& w2, const CSf& w4, int e) {
+    CSf r{(e & 1) ? w1.c : 1.f, (e & 1) ? w1.s : 0.f};
+    const CSf r2 = r.times(w2);
+    if (e & 2) r = r2;
+    const CSf r4 = r.times(w4);
+    if (e & 4) r = r4;
+    return r;
+}
+
+// Coefficients in shared memory, once per block: entry (degree, slot, lane) of
+// the degrees 0..L and the NCH slots a lane uses, the float4 {A, B, S, e}
+// entries first, then the floats f.
+template <int NCH>
+__host__ __device__ constexpr size_t row_table_bytes(int L) {
+    return size_t(L + 1) * NCH * kRowLanes * (sizeof(float4) + sizeof(float));
+}
+
+// Starts the copy of the block's table (16-byte asynchronous copies of the
+// block's threads); row_table_ready() before the first use.
+template <int NCH>
+__device__ __forceinline__ void row_table_load(unsigned char* __restrict__ dst, const float4* __restrict__ rowA,
+                                               const float* __restrict__ rowF, int L) {
+    constexpr int kA = NCH * kRowLanes;      // 16-byte units of one degree: {A, B, S, e}
+    constexpr int kF = NCH * kRowLanes / 4;  // and f
+    const uint32_t sA = smem_u32(dst), sF = sA + uint32_t((L + 1) * kA * 16);
+    for (int i = threadIdx.x; i < (L + 1) * kA; i += blockDim.x)
+        cp_async16(sA + 16 * i, rowA + (i / kA) * (kRowSlots * kRowLanes) + i % kA);
+    const float4* const f4 = reinterpret_cast<const float4*>(rowF);
+    for (int i = threadIdx.x; i < (L + 1) * kF; i += blockDim.x)
+        cp_async16(sF + 16 * i, f4 + (i / kF) * (kRowSlots * kRowLanes / 4) + i % kF);
+}
+__device__ __forceinline__ void row_table_ready() {
+    cp_async_wait_all();
+    __syncthreads();
+}
+
 // Forward kernel. Per degree d and channel slot k (m = j + 8k) a lane runs
-// one step of Eq. iter-q (coefficients from the lane-interleaved table, one
-// degree ahead, so no index arithmetic), then Eq. real-sh-cartesian and
-// Eq. iter-deri for the columns d^2+d+m and d^2+d-m of every plane, stored
-// through per-window plane pointers at compile-time offsets. The m = 0
-// column takes the same path with c_0 = 1/sqrt2 and s_0 = 0 (its -m stores
-// land on the same column first and are overwritten).
-constexpr int kRowMaxWarps = 2;  // warps per block (measured: 1 >= 2 > 4 > 8); the bound frees registers
+// one step of Eq. iter-q, then Eq. real-sh-cartesian and Eq. iter-deri for the
+// columns d^2+d+m and d^2+d-m of every plane, stored through per-window plane
+// pointers at compile-time offsets. The m = 0 column takes the same path with
+// c_0 = 1/sqrt2 and s_0 = 0 (its -m stores land on the same column first and
+// are overwritten).
+//
+// What bounds it: with 8 to 12 warps on an SM (the windows' shared memory), the
+// latency and the number of each slot's instructions. So the coefficients
+// come from shared memory, one slot ahead (from L1, one degree ahead, they
+// cost 1.5 of 5.1 stall cycles per instruction at l_max 50, and the registers
+// that held them one warp in five); one block per SM shares the table. And the
+// derivatives are assembled on the Q side first,
+//   dY/dx = X c_m + q c'_m,  X = x e Q_{d-1}^{m+1} - d u_x q,
+// with c'_m = m c_{m-1} (and 1/r) folded into the kept c_{m-1}: 22 floating-point
+// operations per slot instead of 30.
+constexpr int kRowMaxWarps = 2;  // of an explicit launch shape
+SPH_HD constexpr int row_block_warps(int NCH) { return NCH <= 5 ? 12 : (NCH == 6 ? 10 : (NCH == 7 ? 9 : 8)); }
 
 template <typename TO, bool GRAD, bool NORM, int NCH, bool MINRUN>
-__global__ void __launch_bounds__(32 * kRowMaxWarps) row_fwd_kernel(const float* __restrict__ xyz, int64_t n, int L,
-                                                      const float4* __restrict__ rowA,
+__global__ void __launch_bounds__(32 * row_block_warps(NCH), 1) row_fwd_kernel(const float* __restrict__ xyz, int64_t n,
+                                                      int L, const float4* __restrict__ rowA,
                                                       const float* __restrict__ rowF, float inv_sqrt2,
                                                       TO* __restrict__ sph, TO* __restrict__ dsph) {
     constexpr int NPL = GRAD ? 4 : 1;
     constexpr int SE = RowGeom<TO, NCH, MINRUN>::SE;
     constexpr int BUF = RowGeom<TO, NCH, MINRUN>::BUF;
     constexpr int PSTR = RowGeom<TO, NCH, MINRUN>::template point_stride<NPL>();
+    constexpr int kRow = NCH * kRowLanes;  // table entries of one degree
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int W = blockDim.x >> 5;
     const int g = lane / kG;  // point of the warp tile
     const int j = lane % kG;  // channel class m = j (mod 8)
-    TO* const pst = reinterpret_cast<TO*>(smem) + (size_t(warp) * kPW + g) * PSTR;  // this point's planes
+    row_table_load<NCH>(smem, rowA, rowF, L);
+    const float4* const tA = reinterpret_cast<const float4*>(smem) + j;
+    const float* const tF = reinterpret_cast<const float*>(smem + size_t(L + 1) * kRow * sizeof(float4)) + j;
+    TO* const pst = reinterpret_cast<TO*>(smem + row_table_bytes<NCH>(L)) + (size_t(warp) * kPW + g) * PSTR;
     const int64_t K = int64_t(L + 1) * (L + 1);
     const int64_t ntiles = (n + kPW - 1) / kPW;
     const int nb_lane = (lane & ~(kG - 1)) | ((j + 1) & (kG - 1));  // the lane holding channel m+1's class
-    // this lane's stream: entry (d, k) at laneA[(d * kRowSlots + k) * kRowLanes]
-    const float4* const laneA = rowA + j;
-    const float* const laneF = rowF + j;
+    row_table_ready();
 
     for (int64_t tile = int64_t(blockIdx.x) * W + warp; tile < ntiles; tile += int64_t(gridDim.x) * W) {
         const int64_t p = tile * kPW + g;
@@ -122,27 +173,22 @@ __global__ void __launch_bounds__(32 * kRowMaxWarps) row_fwd_kernel(const float*
         }
         const float r2 = fmaf(z, z, fmaf(x, x, y * y));
 
-        // c_m + i s_m and c_{m-1} + i s_{m-1} of the lane's channels m = j + 8k
+        // c_m + i s_m and m (c_{m-1} + i s_{m-1}) of the lane's channels m = j + 8k
         // (Eq. iter-sc); c_0 carries the 1/sqrt2 of the m = 0 column.
         float cm[NCH], sm[NCH], cm1[NCH], sm1[NCH];
         {
             const CSf xy{x, y};
-            CSf a{1.f, 0.f}, b{1.f, 0.f}, w8{1.f, 0.f}, p7{1.f, 0.f};
-#pragma unroll
-            for (int t = 0; t < kG; ++t) {
-                if (t < j) a = a.times(xy);
-                if (t < j - 1) b = b.times(xy);
-                if (t < kG - 1) p7 = p7.times(xy);
-                w8 = w8.times(xy);
-            }
-            if (j == 0) b = p7;  // channel 8k (k >= 1) needs (x + i y)^(8k-1)
+            const CSf w2 = xy.times(xy), w4 = w2.times(w2), w8 = w4.times(w4);
+            CSf a = row_power(xy, w2, w4, j), b = row_power(xy, w2, w4, (j + kG - 1) % kG);
+            // (for j = 0, b is (x + i y)^7: channel 8k, k >= 1, needs (x + i y)^(8k-1))
 #pragma unroll
             for (int k = 0; k < NCH; ++k) {
                 const bool none = (j == 0 && k == 0);  // m = 0: no c_{m-1}
                 cm[k] = none ? inv_sqrt2 : a.c;
                 sm[k] = none ? 0.f : a.s;
-                cm1[k] = none ? 0.f : b.c;
-                sm1[k] = none ? 0.f : b.s;
+                const float f = NORM ? float(j + kG * k) * ir : float(j + kG * k);
+                cm1[k] = none ? 0.f : f * b.c;  // m c_{m-1} (/ r)
+                sm1[k] = none ? 0.f : f * b.s;
                 a = a.times(w8);
                 if (!none) b = b.times(w8);
             }
@@ -164,16 +210,7 @@ __global__ void __launch_bounds__(32 * kRowMaxWarps) row_fwd_kernel(const float*
             s[i] = (SE - phase) % SE;
         }
 
-        // Degree-0 coefficients; later degrees are loaded one degree ahead.
-        float4 ta[NCH];
-        float tf[NCH];
-#pragma unroll
-        for (int k = 0; k < NCH; ++k) {
-            ta[k] = laneA[k * kRowLanes];
-            tf[k] = laneF[k * kRowLanes];
-        }
         const float xi = NORM ? x * ir : x, yi = NORM ? y * ir : y;
-        const float jf = float(j);
 
         int l = 0;
         bool first = true;
@@ -195,16 +232,8 @@ __global__ void __launch_bounds__(32 * kRowMaxWarps) row_fwd_kernel(const float*
             while (true) {
                 const int ctr = d * d + d;
                 const int kend = d / kG;  // channels m = j + 8k <= d need k <= d/8 (same for the whole warp)
-                const int dn = d < L ? d + 1 : d;
-                // all slots every degree (zeros where m > d): a degree-dependent
-                // bound here keeps more registers live and ran slower
-                float4 na[NCH];
-                float nf[NCH];
-#pragma unroll
-                for (int k = 0; k < NCH; ++k) {  // coefficients of the next degree
-                    na[k] = laneA[(dn * kRowSlots + k) * kRowLanes];
-                    if (GRAD) nf[k] = laneF[(dn * kRowSlots + k) * kRowLanes];
-                }
+                const float4* const dA = tA + d * kRow;
+                const float* const dF = tF + d * kRow;
                 float ax = 0.f, ay = 0.f, az = 0.f;
                 if (NORM && GRAD) {
                     const float lir = float(d) * ir;
@@ -219,45 +248,49 @@ __global__ void __launch_bounds__(32 * kRowMaxWarps) row_fwd_kernel(const float*
                     qp[i] = pp[i] + ctr;
                     qn_[i] = pn[i] + ctr;
                 }
+                // Qtilde_{d-1}^{m+1} of slot k, from the lane that holds channel m + 1
+                auto next_q = [&](int k) {
+                    const float src = (j == 0) ? (k + 1 < NCH ? q1[k + 1 < NCH ? k + 1 : k] : 0.f) : q1[k];
+                    return __shfl_sync(0xffffffffu, src, nb_lane);
+                };
+                float4 tn = dA[0];  // {A, B, S, e} of the next slot
+                float fn = GRAD ? dF[0] : 0.f, qnn = GRAD ? next_q(0) : 0.f;
 #pragma unroll
                 for (int k = 0; k < NCH; ++k) {
                     if (k > kend) break;
-                    const float4 t0 = ta[k];  // {A, B, S, e}
-                    const float src = (j == 0) ? (k + 1 < NCH ? q1[k + 1 < NCH ? k + 1 : k] : 0.f) : q1[k];
-                    const float qnb = __shfl_sync(0xffffffffu, src, nb_lane);  // Qtilde_{l-1}^{m+1}
+                    const float4 t0 = tn;
+                    const float f0 = fn, qnb = qnn;
+                    if (k + 1 < NCH) {
+                        tn = dA[(k + 1) * kRowLanes];
+                        if (GRAD) {
+                            fn = dF[(k + 1) * kRowLanes];
+                            qnn = next_q(k + 1);
+                        }
+                    }
                     // zero for m > d: the table holds zeros there
                     const float q = fmaf(t0.x * z, q1[k], fmaf(-(t0.y * r2), q2[k], t0.z));
                     if (j + kG * k <= d) {
                         const float c = cm[k], sn = sm[k];
-                        const float vc = q * c, vs = q * sn;  // +m (cos) and -m (sin) columns
-                        qn_[0][-kG * k] = OutConv<TO>::cv(vs);
-                        qp[0][kG * k] = OutConv<TO>::cv(vc);
+                        qn_[0][-kG * k] = OutConv<TO>::cv(q * sn);  // -m (sin) and +m (cos) columns
+                        qp[0][kG * k] = OutConv<TO>::cv(q * c);
                         if (GRAD) {
                             // Eq. iter-deri (prefactors folded)
                             const float E1 = t0.w * qnb;  // e Qtilde_{l-1}^{m+1}
-                            const float Qz = NORM ? (tf[k] * q1[k]) * ir : tf[k] * q1[k];
-                            const float Qx = xi * E1, Qy = yi * E1;
-                            const float mQ = (NORM ? (jf + float(kG * k)) * ir : jf + float(kG * k)) * q;
-                            const float mc1 = mQ * cm1[k], ms1 = mQ * sm1[k];
-                            const float tx_c = NORM ? fmaf(-ax, vc, mc1) : mc1;
-                            const float tx_s = NORM ? fmaf(-ax, vs, ms1) : ms1;
-                            const float ty_c = NORM ? fmaf(-ay, vc, -ms1) : -ms1;
-                            const float ty_s = NORM ? fmaf(-ay, vs, mc1) : mc1;
-                            qn_[1 % NPL][-kG * k] = OutConv<TO>::cv(fmaf(Qx, sn, tx_s));
-                            qn_[2 % NPL][-kG * k] = OutConv<TO>::cv(fmaf(Qy, sn, ty_s));
-                            qn_[3 % NPL][-kG * k] = OutConv<TO>::cv(NORM ? fmaf(Qz, sn, -az * vs) : Qz * sn);
-                            qp[1 % NPL][kG * k] = OutConv<TO>::cv(fmaf(Qx, c, tx_c));
-                            qp[2 % NPL][kG * k] = OutConv<TO>::cv(fmaf(Qy, c, ty_c));
-                            qp[3 % NPL][kG * k] = OutConv<TO>::cv(NORM ? fmaf(Qz, c, -az * vc) : Qz * c);
+                            const float Qz = NORM ? (f0 * q1[k]) * ir : f0 * q1[k];
+                            const float X = NORM ? fmaf(-ax, q, xi * E1) : xi * E1;
+                            const float Y = NORM ? fmaf(-ay, q, yi * E1) : yi * E1;
+                            const float Z = NORM ? fmaf(-az, q, Qz) : Qz;
+                            const float mc1 = q * cm1[k], ms1 = q * sm1[k];
+                            qn_[1 % NPL][-kG * k] = OutConv<TO>::cv(fmaf(X, sn, ms1));
+                            qn_[2 % NPL][-kG * k] = OutConv<TO>::cv(fmaf(Y, sn, mc1));
+                            qn_[3 % NPL][-kG * k] = OutConv<TO>::cv(Z * sn);
+                            qp[1 % NPL][kG * k] = OutConv<TO>::cv(fmaf(X, c, mc1));
+                            qp[2 % NPL][kG * k] = OutConv<TO>::cv(fmaf(Y, c, -ms1));
+                            qp[3 % NPL][kG * k] = OutConv<TO>::cv(Z * c);
                         }
                     }
                     q2[k] = q1[k];
                     q1[k] = q;
-                }
-#pragma unroll
-                for (int k = 0; k < NCH; ++k) {
-                    ta[k] = na[k];
-                    if (GRAD) tf[k] = nf[k];
                 }
                 ++d;
                 if (d > L) break;
@@ -356,33 +389,42 @@ __device__ __forceinline__ bool row_window_load(const float* __restrict__ grow, 
     return bulk;
 }
 
+// Like the forward it is bound by the latency and number of each slot's
+// instructions: coefficients from the block's shared table, one slot ahead,
+// and the three sums of point_chan_sums (P = sum e Q_{d-1}^{m+1} A, Bq = sum
+// m Q B, Cq = sum m Q C, with m folded into the kept c_{m-1}), 17
+// floating-point operations per slot where assembling Qx, Qy, Qz took 26. The
+// m = 0 column takes the general path with c_0 = 1/sqrt2, s_0 = 0.
+constexpr int kRowBwdWarps = 16;
+
 template <bool NORM, int NCH>
-__global__ void __launch_bounds__(256) row_bwd_kernel(const float* __restrict__ xyz, const float* __restrict__ g,
-                                                      int64_t n, int L, const float* __restrict__ tb,
-                                                      float inv_sqrt2, float* __restrict__ dxyz,
-                                                      uint32_t* __restrict__ status) {
+__global__ void __launch_bounds__(32 * kRowBwdWarps, 1) row_bwd_kernel(
+    const float* __restrict__ xyz, const float* __restrict__ g, int64_t n, int L, const float4* __restrict__ rowA,
+    const float* __restrict__ rowF, float inv_sqrt2, float* __restrict__ dxyz, uint32_t* __restrict__ status) {
+    constexpr int kRow = NCH * kRowLanes;
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int W = blockDim.x >> 5;
     const int gi = lane / kG;  // point of the warp tile
     const int j = lane % kG;   // channel class m = j (mod 8)
-    unsigned char* wbase = smem + size_t(warp) * row_bwd_warp_bytes();
+    row_table_load<NCH>(smem, rowA, rowF, L);
+    const float4* const tA = reinterpret_cast<const float4*>(smem) + j;
+    const float* const tF = reinterpret_cast<const float*>(smem + size_t(L + 1) * kRow * sizeof(float4)) + j;
+    unsigned char* wbase = smem + row_table_bytes<NCH>(L) + size_t(warp) * row_bwd_warp_bytes();
     float* const bufs = reinterpret_cast<float*>(wbase) + size_t(gi) * 2 * kBBuf;  // this point's two windows
     uint64_t* const bars =
         reinterpret_cast<uint64_t*>(wbase + size_t(kPW) * 2 * kBBuf * sizeof(float)) + 2 * gi;
     const int64_t K = int64_t(L + 1) * (L + 1);
     const int64_t ntiles = (n + kPW - 1) / kPW;
-    const float4* __restrict__ t4 = reinterpret_cast<const float4*>(tb);
     const int nb_lane = (lane & ~(kG - 1)) | ((j + 1) & (kG - 1));
-    const float jf = float(j);
 
     if (j == 0) {
         mbar_init(&bars[0], 1);
         mbar_init(&bars[1], 1);
     }
     fence_proxy_async_smem();
-    __syncwarp();
+    row_table_ready();
     uint32_t parity = 0;   // bit b: phase of buffer b's next completion (same in the 8 lanes of a point)
     uint32_t pending = 0;  // bit b: a bulk load into buffer b is in flight
     bool failed = false;
@@ -409,22 +451,15 @@ __global__ void __launch_bounds__(256) row_bwd_kernel(const float* __restrict__ 
         float cm[NCH], sm[NCH], cm1[NCH], sm1[NCH];
         {
             const CSf xy{x, y};
-            CSf a{1.f, 0.f}, b{1.f, 0.f}, w8{1.f, 0.f}, p7{1.f, 0.f};
-#pragma unroll
-            for (int t = 0; t < kG; ++t) {
-                if (t < j) a = a.times(xy);
-                if (t < j - 1) b = b.times(xy);
-                if (t < kG - 1) p7 = p7.times(xy);
-                w8 = w8.times(xy);
-            }
-            if (j == 0) b = p7;
+            const CSf w2 = xy.times(xy), w4 = w2.times(w2), w8 = w4.times(w4);
+            CSf a = row_power(xy, w2, w4, j), b = row_power(xy, w2, w4, (j + kG - 1) % kG);
 #pragma unroll
             for (int k = 0; k < NCH; ++k) {
-                cm[k] = a.c;
-                sm[k] = a.s;
                 const bool none = (j == 0 && k == 0);
-                cm1[k] = none ? 0.f : b.c;
-                sm1[k] = none ? 0.f : b.s;
+                cm[k] = none ? inv_sqrt2 : a.c;
+                sm[k] = none ? 0.f : a.s;
+                cm1[k] = none ? 0.f : float(j + kG * k) * b.c;  // m c_{m-1}
+                sm1[k] = none ? 0.f : float(j + kG * k) * b.s;
                 a = a.times(w8);
                 if (!none) b = b.times(w8);
             }
@@ -432,14 +467,7 @@ __global__ void __launch_bounds__(256) row_bwd_kernel(const float* __restrict__ 
         float q1[NCH], q2[NCH];
 #pragma unroll
         for (int k = 0; k < NCH; ++k) q1[k] = q2[k] = 0.f;
-        float4 ta[NCH];
-        float tf[NCH];
-#pragma unroll
-        for (int k = 0; k < NCH; ++k) {
-            ta[k] = t4[0];
-            tf[k] = tb[4];
-        }
-        float ax = 0.f, ay = 0.f, az = 0.f, S = 0.f;
+        float P = 0.f, Bq = 0.f, Cq = 0.f, Z = 0.f, S = 0.f;
 
         // window 0 into buffer 0
         int l = 0, lw = row_window_end(0, L), buf = 0;
@@ -470,58 +498,44 @@ __global__ void __launch_bounds__(256) row_bwd_kernel(const float* __restrict__ 
             for (int d = l; d < lw; ++d) {
                 const int ctr = d * d + d;
                 const int kend = d / kG;
-                const int dn = d < L ? d + 1 : L;
-                float4 na[NCH];
-                float nf[NCH];
-#pragma unroll
-                for (int k = 0; k < NCH; ++k) {
-                    const int mk = j + kG * k;
-                    const int i = tri(dn, mk <= dn ? mk : dn);
-                    na[k] = t4[2 * i];
-                    nf[k] = tb[8 * i + 4];
-                }
-                const float lf = float(d);
+                const float4* const dA = tA + d * kRow;
+                const float* const dF = tF + d * kRow;
+                const float* const gp0 = gb + (ctr - s0 + kBPad + j);  // + 8k: g of column ctr + m
+                const float* const gn0 = gb + (ctr - s0 + kBPad - j);
+                float sd = 0.f;
+                auto next_q = [&](int k) {
+                    const float src = (j == 0) ? (k + 1 < NCH ? q1[k + 1 < NCH ? k + 1 : k] : 0.f) : q1[k];
+                    return __shfl_sync(0xffffffffu, src, nb_lane);
+                };
+                float4 tn = dA[0];
+                float fn = dF[0], qnn = next_q(0);
 #pragma unroll
                 for (int k = 0; k < NCH; ++k) {
                     if (k > kend) break;
-                    const int m = j + kG * k;
-                    const bool on = m <= d;
-                    const float4 t0 = ta[k];
-                    const float src = (j == 0) ? (k + 1 < NCH ? q1[k + 1 < NCH ? k + 1 : k] : 0.f) : q1[k];
-                    const float qn = __shfl_sync(0xffffffffu, src, nb_lane);
-                    float q = fmaf(t0.x * z, q1[k], fmaf(-(t0.y * r2), q2[k], t0.z));
-                    q = on ? q : 0.f;
-                    if (on) {
-                        const float E1 = t0.w * qn;
-                        const float Qz = tf[k] * q1[k];
-                        const float Qx = x * E1, Qy = y * E1;
-                        const float gp = gb[ctr + m - s0 + kBPad];
-                        if (k == 0 && j == 0) {  // m = 0: Ytilde_l^0 = Q / sqrt2
-                            ax = fmaf(Qx, gp, ax);
-                            ay = fmaf(Qy, gp, ay);
-                            az = fmaf(Qz, gp, az);
-                            if (NORM) S = fmaf(lf * (q * inv_sqrt2), gp, S);
-                        } else {
-                            const float gn = gb[ctr - m - s0 + kBPad];
-                            const float c = cm[k], sn = sm[k], c1 = cm1[k], s1 = sm1[k];
-                            const float A = fmaf(gp, c, gn * sn);     // g+ c_m + g- s_m
-                            const float B = fmaf(gp, c1, gn * s1);    // g+ c_{m-1} + g- s_{m-1}
-                            const float Cc = fmaf(gn, c1, -(gp * s1));  // g- c_{m-1} - g+ s_{m-1}
-                            const float mQ = (jf + float(kG * k)) * q;
-                            ax = fmaf(Qx, A, fmaf(mQ, B, ax));
-                            ay = fmaf(Qy, A, fmaf(mQ, Cc, ay));
-                            az = fmaf(Qz, A, az);
-                            if (NORM) S = fmaf(lf * q, A, S);
-                        }
+                    const float4 t0 = tn;
+                    const float f0 = fn, qn = qnn;
+                    if (k + 1 < NCH) {
+                        tn = dA[(k + 1) * kRowLanes];
+                        fn = dF[(k + 1) * kRowLanes];
+                        qnn = next_q(k + 1);
+                    }
+                    // zero for m > d: the table holds zeros there
+                    const float q = fmaf(t0.x * z, q1[k], fmaf(-(t0.y * r2), q2[k], t0.z));
+                    if (j + kG * k <= d) {
+                        const float gp = gp0[kG * k], gn = gn0[-kG * k];
+                        const float A = fmaf(gp, cm[k], gn * sm[k]);        // g+ c_m + g- s_m
+                        const float B = fmaf(gp, cm1[k], gn * sm1[k]);      // m (g+ c_{m-1} + g- s_{m-1})
+                        const float Cc = fmaf(gn, cm1[k], -(gp * sm1[k]));  // m (g- c_{m-1} - g+ s_{m-1})
+                        P = fmaf(t0.w * qn, A, P);
+                        Bq = fmaf(q, B, Bq);
+                        Cq = fmaf(q, Cc, Cq);
+                        Z = fmaf(f0 * q1[k], A, Z);
+                        if (NORM) sd = fmaf(q, A, sd);
                     }
                     q2[k] = q1[k];
                     q1[k] = q;
                 }
-#pragma unroll
-                for (int k = 0; k < NCH; ++k) {
-                    ta[k] = na[k];
-                    tf[k] = nf[k];
-                }
+                if (NORM) S = fmaf(float(d), sd, S);
             }
             fence_proxy_async_smem();  // this buffer is rewritten by the async proxy two windows on
             __syncwarp();
@@ -530,6 +544,7 @@ __global__ void __launch_bounds__(256) row_bwd_kernel(const float* __restrict__ 
             buf ^= 1;
         }
         if (failed) break;
+        float ax = fmaf(x, P, Bq), ay = fmaf(y, P, Cq), az = Z;
         // reduce over the 8 lanes of the point
 #pragma unroll
         for (int off = kG / 2; off > 0; off >>= 1) {
@@ -563,10 +578,17 @@ int launch_row(const FwdArgs& a) {
     const float* rt = static_cast<const float*>(device_row_tables());
     if (!rt) return int(cudaErrorMemoryAllocation);
     auto kern = row_fwd_kernel<TO, GRAD, NORM, NCH, MINRUN>;
-    const size_t per_warp = row_warp_bytes<TO, GRAD, NCH, MINRUN>();
-    const int W = a.launch.warps_per_block > 0 ? a.launch.warps_per_block : 1;
+    const size_t per_warp = row_warp_bytes<TO, GRAD, NCH, MINRUN>(), table = row_table_bytes<NCH>(a.l_max);
+    const int64_t tiles = (a.n + kPW - 1) / kPW;
+    int W = a.launch.warps_per_block;
     if (W > kRowMaxWarps) return int(cudaErrorInvalidConfiguration);
-    const size_t smem = size_t(W) * per_warp;
+    if (W <= 0) {
+        // one block per SM with every warp that fits; few tiles are spread over the SMs
+        const int64_t fit = int64_t((size_t(max_smem_optin()) - table) / per_warp);
+        const int64_t spread = (tiles + sm_count() - 1) / sm_count();
+        W = int(std::max<int64_t>(1, std::min<int64_t>({int64_t(row_block_warps(NCH)), fit, spread})));
+    }
+    const size_t smem = table + size_t(W) * per_warp;
     if (smem > size_t(max_smem_optin())) return int(cudaErrorInvalidConfiguration);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kern),
@@ -583,8 +605,7 @@ int launch_row(const FwdArgs& a) {
         }
         bps = std::max(occ, 1);
     }
-    const int64_t ntiles = (a.n + kPW - 1) / kPW;
-    const int64_t want = (ntiles + W - 1) / W;
+    const int64_t want = (tiles + W - 1) / W;
     const int grid = int(std::max<int64_t>(1, std::min<int64_t>(want, int64_t(bps) * sm_count())));
     constexpr int kEntries = kRowLanes * kRowDegrees * kRowSlots;
     kern<<<grid, 32 * W, smem, static_cast<cudaStream_t>(a.stream)>>>(
@@ -594,11 +615,19 @@ int launch_row(const FwdArgs& a) {
 }
 
 template <bool NORM, int NCH>
-int launch_row_bwd(const BwdArgs& a, const float* tb) {
+int launch_row_bwd(const BwdArgs& a) {
+    const float* rt = static_cast<const float*>(device_row_tables());
+    if (!rt) return int(cudaErrorMemoryAllocation);
     auto kern = row_bwd_kernel<NORM, NCH>;
-    const size_t per_warp = row_bwd_warp_bytes();
-    const int W = a.launch.warps_per_block > 0 ? a.launch.warps_per_block : 2;
-    const size_t smem = size_t(W) * per_warp;
+    const size_t per_warp = row_bwd_warp_bytes(), table = row_table_bytes<NCH>(a.l_max);
+    const int64_t tiles = (a.n + kPW - 1) / kPW;
+    int W = a.launch.warps_per_block;
+    if (W <= 0) {
+        const int64_t fit = int64_t((size_t(max_smem_optin()) - table) / per_warp);
+        const int64_t spread = (tiles + sm_count() - 1) / sm_count();
+        W = int(std::max<int64_t>(1, std::min<int64_t>({int64_t(kRowBwdWarps), fit, spread})));
+    }
+    const size_t smem = table + size_t(W) * per_warp;
     if (smem > size_t(max_smem_optin())) return int(cudaErrorInvalidConfiguration);
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kern),
@@ -615,27 +644,28 @@ int launch_row_bwd(const BwdArgs& a, const float* tb) {
         }
         bps = std::max(occ, 1);
     }
-    const int64_t ntiles = (a.n + kPW - 1) / kPW;
-    const int64_t want = (ntiles + W - 1) / W;
+    const int64_t want = (tiles + W - 1) / W;
     const int grid = int(std::max<int64_t>(1, std::min<int64_t>(want, int64_t(bps) * sm_count())));
+    constexpr int kEntries = kRowLanes * kRowDegrees * kRowSlots;
     kern<<<grid, 32 * W, smem, static_cast<cudaStream_t>(a.stream)>>>(
-        static_cast<const float*>(a.xyz), static_cast<const float*>(a.g), a.n, a.l_max, tb,
-        float(host_tables().inv_sqrt2), static_cast<float*>(a.dxyz), a.status);
+        static_cast<const float*>(a.xyz), static_cast<const float*>(a.g), a.n, a.l_max,
+        reinterpret_cast<const float4*>(rt), rt + 4 * kEntries, float(host_tables().inv_sqrt2), static_cast<float*>(a.dxyz), a.status);
     return int(cudaGetLastError());
 }
 
 template <int NCH>
-int launch_row_bwd_flags(const BwdArgs& a, const float* tb) {
-    return a.normalized ? launch_row_bwd<true, NCH>(a, tb) : launch_row_bwd<false, NCH>(a, tb);
+int launch_row_bwd_flags(const BwdArgs& a) {
+    return a.normalized ? launch_row_bwd<true, NCH>(a) : launch_row_bwd<false, NCH>(a);
 }
 
 // Window policy: launch.lanes_per_point 1 = windows that fit the buffer,
 // 2 = windows of at least kCap - SE columns (MINRUN, larger buffers), 0 = by
-// measurement on GB300 (200,000 points, l_max 16..63): FP32 rows keep the
-// smaller buffers (more warps per SM) except at l_max 28..31, where windows
-// that fit fall to ~160 columns (3.26 -> 3.55 TB/s at l_max 30); bf16 rows,
-// half the shared memory, take the longer runs (up to +13 % at l_max 63).
-inline bool row_minrun_default(int L, bool bf16) { return bf16 || (L >= 28 && L <= 31); }
+// measurement on GB300 (60,000..300,000 points): FP32 rows with gradients
+// keep the smaller buffers (more warps per SM), 4..13 % faster, except at l_max
+// 40..52, where windows that fit hold two degrees (l_max 40: 4.92 -> 5.54 TB/s,
+// 46: 4.90 -> 5.34, 50: 5.00 -> 5.18, 54: 4.87 -> 4.59); bf16 rows, half the
+// shared memory, take the longer runs (up to +13 % at l_max 63).
+inline bool row_minrun_default(int L, bool bf16) { return bf16 || (L >= 40 && L <= 52); }
 
 template <typename TO, int NCH, bool MINRUN>
 int launch_row_policy(const FwdArgs& a) {
@@ -662,15 +692,13 @@ int launch_row_out(const FwdArgs& a) {
 
 #if SPH_ROW_PART == 0
 int row_bwd_part0(const BwdArgs& a) {
-    const float* tb = static_cast<const float*>(device_tables(SPH_F32));
-    if (!tb) return int(cudaErrorMemoryAllocation);
     switch ((a.l_max + 1 + kG - 1) / kG) {
         case 3:
-            return launch_row_bwd_flags<3>(a, tb);
+            return launch_row_bwd_flags<3>(a);
         case 4:
-            return launch_row_bwd_flags<4>(a, tb);
+            return launch_row_bwd_flags<4>(a);
         default:
-            return launch_row_bwd_flags<5>(a, tb);
+            return launch_row_bwd_flags<5>(a);
     }
 }
 
@@ -686,15 +714,13 @@ int row_fwd_part0(const FwdArgs& a) {
 }
 #else
 int row_bwd_part1(const BwdArgs& a) {
-    const float* tb = static_cast<const float*>(device_tables(SPH_F32));
-    if (!tb) return int(cudaErrorMemoryAllocation);
     switch ((a.l_max + 1 + kG - 1) / kG) {
         case 6:
-            return launch_row_bwd_flags<6>(a, tb);
+            return launch_row_bwd_flags<6>(a);
         case 7:
-            return launch_row_bwd_flags<7>(a, tb);
+            return launch_row_bwd_flags<7>(a);
         default:
-            return launch_row_bwd_flags<8>(a, tb);
+            return launch_row_bwd_flags<8>(a);
     }
 }
 
