@@ -1014,35 +1014,123 @@ __device__ __forceinline__ int64_t issue_tile_load(T* dst, const T* src, int64_t
 
 constexpr uint32_t kWaitPolls = 1u << 22;  // bounded mbarrier wait (>> any real load latency)
 
-template <typename T, bool NORM, int K>
-struct BwdVis {
-    const T* gr;  // this lane's upstream-gradient row in shared memory
-    T ax, ay, az, S;
-    __device__ __forceinline__ void emit(int l, int k, const Deriv<T>& d) {
-        const T gk = gr[k];
-        ax += gk * d.gx;
-        ay += gk * d.gy;
-        az += gk * d.gz;
-        if (NORM) S += gk * (T(l) * d.v);
-    }
+// Sums over all columns of one point, sum_k g_k dY_k/dx_i, channel by channel.
+// The columns +-m of degree l enter only through three combinations of the
+// two upstream gradients,
+//   A = g+ c_m + g- s_m,  B = g+ c_{m-1} + g- s_{m-1},  C = g- c_{m-1} - g+ s_{m-1},
+// and the terms of Eq. iter-deri, summed over (l, m), are
+//   P = sum e Q_{l-1}^{m+1} A,  Bq = sum m Q B,  Cq = sum m Q C,  Z = sum f Q_{l-1}^m A
+// (Q = Qtilde_l^m, Q_{l-1} = Qtilde_{l-1}): the gradient is (x P + Bq, y P + Cq, Z).
+// With DUAL the same sums are differentiated along the direction (dx, dy, dz):
+//   dQ_l^m = (x dx + y dy) e Q_{l-1}^{m+1} + dz f Q_{l-1}^m,
+//   dA = m (dx B + dy C),  dB, dC from dc_{m-1}, ds_{m-1} likewise,
+// and every column's own derivative along that direction, dQ c_m + Q dc_m and
+// dQ s_m + Q ds_m, replaces its upstream gradient's slot in `orow`. That is
+// the double backward (grad_xyz is the derivative of the gradient along v,
+// grad_g the derivative of Y along v) without any Hessian entry: 37 operations
+// per pair of columns (17 without DUAL) where the six Hessian entries of both
+// columns and their products with g and v took about 130 (27).
+// S = sum l Y g is the term of the normalized form.
+template <typename T>
+struct ChanSums {
+    T P = T(0), Bq = T(0), Cq = T(0), Z = T(0), S = T(0);
+    T dP = T(0), dB = T(0), dC = T(0), dZ = T(0), dS = T(0);
 };
 
-template <typename T, bool NORM, int K>
-struct DbwdVis {
-    const T* gr;  // upstream gradient row (shared)
-    T* orow;      // grad_g row (shared)
-    T vx, vy, vz;
-    T ux, uy, uz, ir;
-    T ax, ay, az;
-    __device__ __forceinline__ void emit(int l, int k, Deriv<T> d) {
-        if (NORM) normalize_deriv<true>(d, l, ux, uy, uz, ir);
-        const T gk = gr[k];
-        orow[k] = vx * d.gx + vy * d.gy + vz * d.gz;
-        ax += gk * (d.hxx * vx + d.hxy * vy + d.hxz * vz);
-        ay += gk * (d.hxy * vx + d.hyy * vy + d.hyz * vz);
-        az += gk * (d.hxz * vx + d.hyz * vy + d.hzz * vz);
+template <int L, bool NORM, bool DUAL, typename T, typename Tabs>
+__device__ __forceinline__ void point_chan_sums(T x, T y, T z, T r2, T dx, T dy, T dz, const Tabs& tb,
+                                                const T* __restrict__ gr, T* __restrict__ orow, ChanSums<T>& a) {
+    T c[L + 1], s[L + 1];
+    point_cs<L>(x, y, c, s);
+    const T w = DUAL ? x * dx + y * dy : T(0);
+    T q1[L + 1], q2[L + 1], p1[L + 1];  // Qtilde_{l-1}^m, Qtilde_{l-2}^m, (DUAL) d Qtilde_{l-1}^m
+#pragma unroll
+    for (int m = 0; m <= L; ++m) q1[m] = q2[m] = p1[m] = T(0);
+#pragma unroll
+    for (int l = 0; l <= L; ++l) {
+        T q[L + 1], p[L + 1];
+        q[l] = tb.qll[l];
+        if (l >= 1) q[l - 1] = tb.d[l] * z * q1[l - 1];
+#pragma unroll
+        for (int m = 0; m + 2 <= l; ++m) {  // Eq. iter-q, folded
+            const int i = tri(l, m);
+            q[m] = (tb.a[i] * z) * q1[m] - (tb.b[i] * r2) * q2[m];
+        }
+        T sl = T(0), dsl = T(0);  // sum over the degree of Y g, and its derivative
+#pragma unroll
+        for (int m = 0; m <= l; ++m) {
+            const int i = tri(l, m);
+            const T E1 = (m + 1 <= l - 1) ? tb.e[i] * q1[m + 1] : T(0);
+            const T Qz = (m <= l - 1) ? tb.fz[i] * q1[m] : T(0);
+            // the multipliers of the m = 0 column carry its 1/sqrt2
+            T dE1 = T(0), dQz = T(0), dq = T(0);
+            if constexpr (DUAL) {
+                dE1 = (m + 1 <= l - 1) ? tb.e[i] * p1[m + 1] : T(0);
+                dQz = (m <= l - 1) ? tb.fz[i] * p1[m] : T(0);
+                dq = w * E1 + dz * Qz;
+            }
+            const int k = l * l + l;
+            if (m == 0) {
+                const T g = gr[k];
+                a.P += E1 * g;
+                a.Z += Qz * g;
+                if (NORM) sl += (tb.inv_sqrt2 * q[0]) * g;
+                if constexpr (DUAL) {
+                    orow[k] = dq;
+                    a.dP += dE1 * g;
+                    a.dZ += dQz * g;
+                    if (NORM) dsl += dq * g;
+                    p[0] = dq * (T(2) * tb.inv_sqrt2);
+                }
+            } else {
+                const T gp = gr[k + m], gn = gr[k - m];
+                const T c1 = c[m - 1], s1 = s[m - 1];
+                const T A = gp * c[m] + gn * s[m];
+                const T B = gp * c1 + gn * s1;
+                const T C = gn * c1 - gp * s1;
+                const T mq = T(m) * q[m];
+                a.P += E1 * A;
+                a.Z += Qz * A;
+                if (NORM || !DUAL) {  // the gradient itself
+                    a.Bq += mq * B;
+                    a.Cq += mq * C;
+                }
+                if (NORM) sl += q[m] * A;
+                if constexpr (DUAL) {
+                    const T mx = T(m) * dx, my = T(m) * dy;
+                    const T dcm = mx * c1 - my * s1, dsm = mx * s1 + my * c1;
+                    orow[k + m] = dq * c[m] + q[m] * dcm;
+                    orow[k - m] = dq * s[m] + q[m] * dsm;
+                    const T dA = mx * B + my * C;
+                    const T mdq = T(m) * dq;
+                    a.dP += dE1 * A + E1 * dA;
+                    a.dZ += dQz * A + Qz * dA;
+                    a.dB += mdq * B;
+                    a.dC += mdq * C;
+                    if (m >= 2) {
+                        const T c2 = c[m >= 2 ? m - 2 : 0], s2 = s[m >= 2 ? m - 2 : 0];
+                        const T nx = T(m - 1) * dx, ny = T(m - 1) * dy;
+                        const T dc1 = nx * c2 - ny * s2, ds1 = nx * s2 + ny * c2;
+                        a.dB += mq * (gp * dc1 + gn * ds1);
+                        a.dC += mq * (gn * dc1 - gp * ds1);
+                    }
+                    if (NORM) dsl += dq * A + q[m] * dA;
+                    p[m] = dq;
+                }
+            }
+        }
+        if (NORM) {
+            a.S += T(l) * sl;
+            if (DUAL) a.dS += T(l) * dsl;
+        }
+#pragma unroll
+        for (int m = 0; m <= l; ++m) {
+            q2[m] = q1[m];
+            q1[m] = q[m];
+            if (DUAL) p1[m] = p[m];
+        }
     }
-};
+}
 
 template <int L, typename T>
 __host__ __device__ constexpr size_t point_bwd_buf_bytes(int P) {
@@ -1055,7 +1143,7 @@ __host__ __device__ constexpr size_t point_bwd_buf_bytes(int P) {
 template <int L, bool NORM, bool DBW, typename T>
 __global__ void __launch_bounds__(256) point_bwd_kernel(const T* __restrict__ xyz, const T* __restrict__ g,
                                                         const T* __restrict__ v, int64_t n,
-                                                        const __grid_constant__ PointTabs<L, T, DBW> tb,
+                                                        const __grid_constant__ PointTabs<L, T, false> tb,
                                                         T* __restrict__ dxyz, T* __restrict__ grad_g,
                                                         T* __restrict__ grad_xyz, int P, int bulk_in,
                                                         int bulk_out, uint32_t* __restrict__ status) {
@@ -1143,36 +1231,46 @@ __global__ void __launch_bounds__(256) point_bwd_kernel(const T* __restrict__ xy
             } else {
                 r2 = x * x + y * y + z * z;
             }
+            const T* gr = gt + size_t(lane) * RS::V;
+            ChanSums<T> a;
             if constexpr (!DBW) {
-                BwdVis<T, NORM, K> vis{gt + size_t(lane) * RS::V, T(0), T(0), T(0), T(0)};
-                point_core<L, true, false>(x, y, z, r2, tb, vis);
-                T ax = vis.ax, ay = vis.ay, az = vis.az;
+                point_chan_sums<L, NORM, false>(x, y, z, r2, T(0), T(0), T(0), tb, gr, static_cast<T*>(nullptr), a);
+                T ax = x * a.P + a.Bq, ay = y * a.P + a.Cq, az = a.Z;
                 if (NORM) {
-                    ax = ir * (ax - x * vis.S);
-                    ay = ir * (ay - y * vis.S);
-                    az = ir * (az - z * vis.S);
+                    ax = ir * (ax - x * a.S);
+                    ay = ir * (ay - y * a.S);
+                    az = ir * (az - z * a.S);
                 }
                 dxyz[3 * p] = ax;
                 dxyz[3 * p + 1] = ay;
                 dxyz[3 * p + 2] = az;
             } else {
-                DbwdVis<T, NORM, K> vis{gt + size_t(lane) * RS::V,
-                                        so + size_t(lane) * RS::V,
-                                        v[3 * p],
-                                        v[3 * p + 1],
-                                        v[3 * p + 2],
-                                        x,
-                                        y,
-                                        z,
-                                        ir,
-                                        T(0),
-                                        T(0),
-                                        T(0)};
-                point_core<L, true, true>(x, y, z, r2, tb, vis);
+                // direction of the derivative at the evaluated point: v, or
+                // (normalized) that of u = x / r, (v - u (u.v)) / r
+                T dx = v[3 * p], dy = v[3 * p + 1], dz = v[3 * p + 2], uv = T(0);
+                if (NORM) {
+                    uv = x * dx + y * dy + z * dz;
+                    dx = ir * (dx - x * uv);
+                    dy = ir * (dy - y * uv);
+                    dz = ir * (dz - z * uv);
+                }
+                point_chan_sums<L, NORM, true>(x, y, z, r2, dx, dy, dz, tb, gr, so + size_t(lane) * RS::V, a);
                 if (grad_xyz) {
-                    grad_xyz[3 * p] = vis.ax;
-                    grad_xyz[3 * p + 1] = vis.ay;
-                    grad_xyz[3 * p + 2] = vis.az;
+                    T hx = dx * a.P + x * a.dP + a.dB;
+                    T hy = dy * a.P + y * a.dP + a.dC;
+                    T hz = a.dZ;
+                    if (NORM) {  // of (1/r) (G - u S): d(1/r) = -(u.v) / r^2
+                        const T gx = x * a.P + a.Bq - x * a.S;
+                        const T gy = y * a.P + a.Cq - y * a.S;
+                        const T gz = a.Z - z * a.S;
+                        const T iu = ir * uv;
+                        hx = ir * (hx - dx * a.S - x * a.dS - iu * gx);
+                        hy = ir * (hy - dy * a.S - y * a.dS - iu * gy);
+                        hz = ir * (hz - dz * a.S - z * a.dS - iu * gz);
+                    }
+                    grad_xyz[3 * p] = hx;
+                    grad_xyz[3 * p + 1] = hy;
+                    grad_xyz[3 * p + 2] = hz;
                 }
             }
         }
@@ -1364,7 +1462,7 @@ int launch_point10_fwd(const FwdArgs& a) {
 
 template <int L, bool NORM, bool DBW, typename T>
 int launch_point_bwd(const BwdArgs& a) {
-    static const PointTabs<L, T, DBW> tb = make_point_tabs<L, T, DBW>();
+    static const PointTabs<L, T, false> tb = make_point_tabs<L, T, false>();
     const int P = a.launch.points_per_tile, W = a.launch.warps_per_block;
     const size_t smem = size_t(W) * ((DBW ? 3 : 2) * point_bwd_buf_bytes<L, T>(P) + 16);
     auto kern = point_bwd_kernel<L, NORM, DBW, T>;
