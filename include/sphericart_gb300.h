@@ -80,7 +80,8 @@ typedef enum { SPH_Q_NATIVE = 0, SPH_Q_F64 = 1 } sph_qprec;
 /* Kernel family. AUTO picks, by measurement on GB300: DEGREE for FP64
  * arithmetic without Hessians (the mixed mode; SPH_F64 from l_max 14, with
  * gradients from l_max 9); else
- * ROW for FP32 Hessians with FP32 storage up to l_max 63, from l_max 14 in
+ * ROW for FP32 Hessians with FP32 storage up to l_max 63, from l_max 16
+ * (below 8,192 points 14) in
  * the normalized form and beyond SPH_MAX_L_POINT in the scaled one
  * (launch_info reports the scaled form's choice); else POINT when
  * l_max <= SPH_MAX_L_POINT (except bfloat16 Hessians); else ROW for FP32
@@ -154,7 +155,7 @@ typedef enum {
  * bf16) or up to 32 points in <= 74 KB with one warp per block (FP64, bound by
  * the FP64 pipe), and with FP32 gradients from l_max 10 runs 4 lanes per
  * point on 8-point tiles, with FP32 Hessians 10 lanes per point where that
- * measured faster (scaled l_max 7..16, normalized 6..13; ROW above); when a call
+ * measured faster (scaled l_max 7..16, normalized 6..15; ROW above); when a call
  * has fewer than 2 x SMs x
  * warps_per_block tiles, it runs fewer warps per block so that the blocks
  * reach every SM.                                                           */

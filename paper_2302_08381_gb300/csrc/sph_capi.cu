@@ -344,8 +344,8 @@ sph_launch default_point10_fwd(int L) {
 // (1.1x the 16-lane map at l_max 8, 2.3x at 11, 3.6x at 16) and for the
 // normalized form from l_max 6 (1.2-1.6x); the one-lane tile is faster below;
 // AUTO runs ROW from row_hess_min_auto.
-bool point10_default(int L, int hess, int normalized, int dtype, int out) {
-    if (!hess || dtype != SPH_F32 || out != SPH_OUT_SAME || L >= row_hess_min_auto(normalized)) return false;
+bool point10_default(int L, int hess, int normalized, int dtype, int out, int64_t n) {
+    if (!hess || dtype != SPH_F32 || out != SPH_OUT_SAME || L >= row_hess_min_auto(normalized, n)) return false;
     return L >= (normalized ? 6 : 7);
 }
 
@@ -501,15 +501,15 @@ namespace {
 // lanes) is fastest; beyond POINT's range FP32 arithmetic runs on ROW up to
 // its l_max 63 (1.8-2.2x SLICE; FP32 Hessians 1.2-1.7x), then on SLICE
 // (DEGREE for bf16 storage).
-int auto_family(int l_max, int dtype, int out, int qprec, bool hess, bool grad, int normalized) {
+int auto_family(int l_max, int dtype, int out, int qprec, bool hess, bool grad, int normalized, int64_t n) {
     const bool mixed = dtype == SPH_F32 && qprec == SPH_Q_F64;
     // FP64: DEGREE with gradients from l_max 9 (measured at 1M-4M points:
     // l_max 10 / 11 at 1.65x / 2.0x POINT), values from l_max 14 (POINT 8 %
     // faster at l_max 12, equal at 13; at 10k points POINT up to 16)
     if (!hess && (mixed || (dtype == SPH_F64 && (l_max >= 14 || (grad && l_max >= 9))))) return SPH_KERNEL_DEGREE;
     if (!hess && point_hybrid_wins(l_max, dtype, grad)) return SPH_KERNEL_POINT_HC;
-    // FP32 Hessians: ROW from l_max 13 (normalized) or beyond POINT's range
-    if (hess && dtype == SPH_F32 && out == SPH_OUT_SAME && l_max >= row_hess_min_auto(normalized) &&
+    // FP32 Hessians: ROW from row_hess_min_auto (normalized) or beyond POINT's range
+    if (hess && dtype == SPH_F32 && out == SPH_OUT_SAME && l_max >= row_hess_min_auto(normalized, n) &&
         l_max <= kRowMaxL)
         return SPH_KERNEL_ROW;
     if (l_max <= SPH_MAX_L_POINT && !(hess && out == SPH_OUT_BF16)) return SPH_KERNEL_POINT;
@@ -615,7 +615,7 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
     int fam = kernel;
     const bool hess_bf16 = ddsph && out == SPH_OUT_BF16;
     if (fam == SPH_KERNEL_AUTO)
-        fam = auto_family(l_max, dtype, out, qprec, ddsph != nullptr, dsph != nullptr, normalized);
+        fam = auto_family(l_max, dtype, out, qprec, ddsph != nullptr, dsph != nullptr, normalized, n);
     int hc = 0;
     if (fam == SPH_KERNEL_POINT_HC) {
         if (l_max > kHcMaxL || ddsph || mixed || out != SPH_OUT_SAME) {
@@ -676,7 +676,7 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
             a.launch.blocks_per_sm == 0 && a.launch.lanes_per_point == 0) {
             if (point4_default(l_max, grad, eo, hess, hc))
                 a.launch.lanes_per_point = 4;
-            else if (point10_default(l_max, hess, normalized, dtype, out))
+            else if (point10_default(l_max, hess, normalized, dtype, out, n))
                 a.launch.lanes_per_point = 10;
         }
         const int lpp = a.launch.lanes_per_point;
@@ -909,7 +909,7 @@ int sphericart_launch_info(int l_max, int dtype, int out, int grad, int hess, in
         return SPH_EINVAL;
     }
     const int eo = elem_size(dtype, out);
-    int fam = auto_family(l_max, dtype, out, SPH_Q_NATIVE, hess != 0, grad != 0, 0);  // (the scaled form's choice)
+    int fam = auto_family(l_max, dtype, out, SPH_Q_NATIVE, hess != 0, grad != 0, 0, 0);  // (the scaled form's choice)
     const bool hc = fam == SPH_KERNEL_POINT_HC;
     if (hc) fam = SPH_KERNEL_POINT;  // same launch shapes
     if (fam == SPH_KERNEL_DEGREE) {
@@ -935,7 +935,7 @@ int sphericart_launch_info(int l_max, int dtype, int out, int grad, int hess, in
                           s.lanes_per_point == 0;
         const bool four = s.lanes_per_point == 4 || (none && point4_default(l_max, grad, eo, hess, hc ? 1 : 0));
         // (the scaled form's choice: launch_info takes no normalized flag)
-        const bool ten = s.lanes_per_point == 10 || (none && !four && point10_default(l_max, hess, 0, dtype, out));
+        const bool ten = s.lanes_per_point == 10 || (none && !four && point10_default(l_max, hess, 0, dtype, out, 0));
         const bool sixteen = s.lanes_per_point == 16;
         const sph_launch dflt = four      ? default_point4_fwd(l_max, eo)
                                 : ten     ? default_point10_fwd(l_max)

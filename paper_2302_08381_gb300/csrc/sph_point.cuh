@@ -566,12 +566,15 @@ __global__ void __launch_bounds__(256) point4_fwd_kernel(const T* __restrict__ x
 //   B = bQ Qtilde + bE e Qtilde_{l-1}^{m+1} + bz f Qtilde_{l-1}^m
 // with C = c_m (or s_m for the sin-type column), T1 a role combination of
 // c_{m-1}, s_{m-1} and T2 of c_{m-2}, s_{m-2} (the derivatives of c_m, s_m),
-// role weights from the point's coordinates. The normalized form needs the
-// value and two gradient components of the same column: taken from the
-// point's lanes 0 and 1 + i by warp shuffles.
+// role weights from the point's coordinates. The normalized form,
+//   sc (plane + wv Y - l u_k g_i - l u_i g_k),  g_i = X_i e Qtilde_{l-1}^{m+1} C + ... + m Qtilde_l^m T_i,
+// is linear in the same terms, so it only changes the weights with l (aQ, aE,
+// az) and adds l m Qtilde_l^m T3, T3 a role combination of c_{m-1}, s_{m-1}: one
+// fma more per column. (Taking Y, g_i and g_k of the column from the lanes that
+// own those planes cost six shuffles and eight operations per pair of columns.)
 template <int L, bool NORM, bool TWO = false, typename Tabs>
-__device__ __forceinline__ void point16_core(float x, float y, float z, float r2, const Tabs& tb, int rr, int base,
-                                             float ir, float* __restrict__ rowp, float* __restrict__ rowp2,
+__device__ __forceinline__ void point16_core(float x, float y, float z, float r2, const Tabs& tb, int rr, float ir,
+                                             float* __restrict__ rowp, float* __restrict__ rowp2,
                                              bool store) {
     const int hi = rr >= 4 ? (rr - 4) / 3 : 0, hk = rr >= 4 ? (rr - 4) % 3 : 0;
     // the symmetric entry (i, k) with i <= k selects the formula
@@ -580,15 +583,17 @@ __device__ __forceinline__ void point16_core(float x, float y, float z, float r2
     const bool hxx = ish && i0 == 0 && k0 == 0, hxy = ish && i0 == 0 && k0 == 1, hxz = ish && i0 == 0 && k0 == 2;
     const bool hyy = ish && i0 == 1 && k0 == 1, hyz = ish && i0 == 1 && k0 == 2, hzz = ish && i0 == 2 && k0 == 2;
     const float X = x, Y = y;
+    // scale of the plane: 1/r of the gradient, 1/r^2 of the Hessian (normalized)
+    const float sc = !NORM || isv ? 1.f : (ish ? ir * ir : ir);
     const float aQ = isv ? 1.f : 0.f;
-    const float aE = isgx ? X : (isgy ? Y : ((hxx || hyy) ? 1.f : 0.f));
-    const float az = isgz ? 1.f : 0.f;
-    const float a2 = hxx ? X * X : (hyy ? Y * Y : (hxy ? X * Y : 0.f));
-    const float a3 = hxz ? X : (hyz ? Y : 0.f);
-    const float a4 = hzz ? 1.f : 0.f;
-    const float bQ = (isgx || isgy) ? 1.f : 0.f;
-    const float bE = (hxx || hyy || hxy) ? 1.f : 0.f;
-    const float bz = (hxz || hyz) ? 1.f : 0.f;
+    const float aE = sc * (isgx ? X : (isgy ? Y : ((hxx || hyy) ? 1.f : 0.f)));
+    const float az = sc * (isgz ? 1.f : 0.f);
+    const float a2 = sc * (hxx ? X * X : (hyy ? Y * Y : (hxy ? X * Y : 0.f)));
+    const float a3 = sc * (hxz ? X : (hyz ? Y : 0.f));
+    const float a4 = sc * (hzz ? 1.f : 0.f);
+    const float bQ = (isgx || isgy) ? sc : 0.f;
+    const float bE = (hxx || hyy || hxy) ? sc : 0.f;
+    const float bz = (hxz || hyz) ? sc : 0.f;
     // T1c = k1c c1 + k1s s1, T1s = k2c c1 + k2s s1, T2c = k3c c2 + k3s s2, T2s = k4c c2 + k4s s2
     float k1c = 0.f, k1s = 0.f, k2c = 0.f, k2s = 0.f, k3c = 0.f, k3s = 0.f, k4c = 0.f, k4s = 0.f;
     if (isgx || hxz) {
@@ -600,32 +605,39 @@ __device__ __forceinline__ void point16_core(float x, float y, float z, float r2
     } else if (hxx) {
         k1c = 2.f * X;
         k2s = 2.f * X;
-        k3c = 1.f;
-        k4s = 1.f;
+        k3c = sc;
+        k4s = sc;
     } else if (hyy) {
         k1s = -2.f * Y;
         k2c = 2.f * Y;
-        k3c = -1.f;
-        k4s = -1.f;
+        k3c = -sc;
+        k4s = -sc;
     } else if (hxy) {
         k1c = Y;
         k1s = -X;
         k2c = X;
         k2s = Y;
-        k3s = -1.f;
-        k4c = 1.f;
+        k3s = -sc;
+        k4c = sc;
     }
     float c[L + 1], s[L + 1];
     point_cs<L>(x, y, c, s);
-    // Normalized form: plane' = sc (plane + wv v + wi g_i + wk g_k), v and g from
-    // the point's lanes 0 and 1 + i / 1 + k (raw values at the unit point).
-    // (i0, k0) for both (i, k) and (k, i): the two planes of a symmetric pair
-    // run the same operations and come out bit-identical; `base` is the lane
-    // of the point's value plane, base + 1 + i that of gradient component i
-    const int src_i = base + 1 + i0, src_k = base + 1 + k0;
+    // Normalized form, (i0, k0) for both (i, k) and (k, i): the two planes of a
+    // symmetric pair run the same operations and come out bit-identical.
+    // Weights of l (l (l + 2) for nv2) in aQ, aE and az, and of l m Qtilde in T3
     const float ui = i0 == 0 ? x : (i0 == 1 ? y : z), uk = k0 == 0 ? x : (k0 == 1 ? y : z);
-    const float ug = isgx ? x : (isgy ? y : z);  // gradient planes: u of their component
-    const float sc = !NORM || isv ? 1.f : (ish ? ir * ir : ir);
+    float nv = 0.f, nv2 = 0.f, nE = 0.f, nz = 0.f, k5 = 0.f, k6 = 0.f;
+    if (NORM && ish) {
+        const float si = -sc * uk, sk = -sc * ui;
+        nv = i0 == k0 ? -sc : 0.f;
+        nv2 = sc * ui * uk;
+        k5 = (i0 == 0 ? si : 0.f) + (k0 == 0 ? sk : 0.f);  // T3c = k5 c1 - k6 s1, T3s = k5 s1 + k6 c1
+        k6 = (i0 == 1 ? si : 0.f) + (k0 == 1 ? sk : 0.f);
+        nE = k5 * X + k6 * Y;
+        nz = (i0 == 2 ? si : 0.f) + (k0 == 2 ? sk : 0.f);
+    } else if (NORM && !isv) {
+        nv = -sc * (isgx ? x : (isgy ? y : z));
+    }
     float q1[L + 1], q2[L + 1];
 #pragma unroll
     for (int m = 0; m <= L; ++m) {
@@ -642,18 +654,9 @@ __device__ __forceinline__ void point16_core(float x, float y, float z, float r2
             const int i = tri(l, m);
             q[m] = (tb.a[i] * z) * q1[m] - (tb.b[i] * r2) * q2[m];
         }
-        const float lf = float(l);
-        // normalization weights of this degree
-        float wv = 0.f, wi = 0.f, wk = 0.f;
-        if (NORM) {
-            if (ish) {
-                wv = lf * (lf + 2.f) * ui * uk - (i0 == k0 ? lf : 0.f);
-                wi = -lf * uk;
-                wk = -lf * ui;
-            } else if (!isv) {
-                wv = -lf * ug;
-            }
-        }
+        const float aQl = NORM ? fmaf(float(l * (l + 2)), nv2, fmaf(float(l), nv, aQ)) : aQ;
+        const float aEl = NORM ? fmaf(float(l), nE, aE) : aE;
+        const float azl = NORM ? fmaf(float(l), nz, az) : az;
 #pragma unroll
         for (int m = 0; m <= l; ++m) {
             const int i = tri(l, m);
@@ -662,40 +665,30 @@ __device__ __forceinline__ void point16_core(float x, float y, float z, float r2
             const float G2 = (m + 2 <= l - 2) ? tb.g2[i] * q2[m + 2] : 0.f;
             const float G3 = (m + 1 <= l - 2) ? tb.g3[i] * q2[m + 1] : 0.f;
             const float G4 = (m <= l - 2) ? tb.g4[i] * q2[m] : 0.f;
-            const float A = aE * E1 + az * Qz + a2 * G2 + a3 * G3 + a4 * G4;
+            const float A = aEl * E1 + azl * Qz + a2 * G2 + a3 * G3 + a4 * G4;
             if (m == 0) {
-                float out = aQ * tb.inv_sqrt2 * q[0] + A;
-                if (NORM) {
-                    const float v = __shfl_sync(0xffffffffu, out, base);
-                    const float gi = __shfl_sync(0xffffffffu, out, src_i);
-                    const float gk = __shfl_sync(0xffffffffu, out, src_k);
-                    out = sc * (out + wv * v + wi * gi + wk * gk);
-                }
+                const float out = aQl * tb.inv_sqrt2 * q[0] + A;
                 if (store) {
                     rowp[l * l + l] = out;
                     if (TWO) rowp2[l * l + l] = out;
                 }
             } else {
-                const float Am = aQ * q[m] + A;
+                const float Am = aQl * q[m] + A;
                 const float mB = float(m) * (bQ * q[m] + bE * E1 + bz * Qz);
-                const float MQ = float(m * (m - 1)) * q[m];
+                const float mq = float(m) * q[m];
                 const float c1 = c[m - 1], s1 = s[m - 1];
                 const float c2 = m >= 2 ? c[m >= 2 ? m - 2 : 0] : 0.f, s2 = m >= 2 ? s[m >= 2 ? m - 2 : 0] : 0.f;
                 float oc = Am * c[m] + mB * (k1c * c1 + k1s * s1);
                 float os = Am * s[m] + mB * (k2c * c1 + k2s * s1);
-                if (m >= 2) {
+                if (NORM) {
+                    const float Uc = float(l) * (k5 * c1 - k6 * s1) + float(m - 1) * (k3c * c2 + k3s * s2);
+                    const float Us = float(l) * (k5 * s1 + k6 * c1) + float(m - 1) * (k4c * c2 + k4s * s2);
+                    oc += mq * Uc;
+                    os += mq * Us;
+                } else if (m >= 2) {
+                    const float MQ = float(m - 1) * mq;
                     oc += MQ * (k3c * c2 + k3s * s2);
                     os += MQ * (k4c * c2 + k4s * s2);
-                }
-                if (NORM) {
-                    const float vc = __shfl_sync(0xffffffffu, oc, base);
-                    const float gic = __shfl_sync(0xffffffffu, oc, src_i);
-                    const float gkc = __shfl_sync(0xffffffffu, oc, src_k);
-                    const float vs = __shfl_sync(0xffffffffu, os, base);
-                    const float gis = __shfl_sync(0xffffffffu, os, src_i);
-                    const float gks = __shfl_sync(0xffffffffu, os, src_k);
-                    oc = sc * (oc + wv * vc + wi * gic + wk * gkc);
-                    os = sc * (os + wv * vs + wi * gis + wk * gks);
                 }
                 if (store) {
                     rowp[l * l + l + m] = oc;
@@ -767,7 +760,7 @@ __device__ __forceinline__ void point16_tile(const float* __restrict__ xyz, floa
         const int rr = r < 13 ? r : 12;
         float* rowp = rr == 0 ? s_v + size_t(j) * S
                               : (rr < 4 ? s_d + size_t(3 * j + rr - 1) * S : s_h + size_t(9 * j + rr - 4) * S);
-        point16_core<L, NORM>(x, y, z, r2, tb, rr, lane & 16, ir, rowp, rowp, r < 13);
+        point16_core<L, NORM>(x, y, z, r2, tb, rr, ir, rowp, rowp, r < 13);
         if constexpr (MODE == 1) {
             if (bulk && r < 13 && j < cnt) {  // each lane sends the row it wrote
                 fence_proxy_async_smem();
@@ -925,10 +918,10 @@ __device__ __forceinline__ void point10_tile(const float* __restrict__ xyz, floa
             float* rowp = rr == 0 ? iv + size_t(pj) * S
                                   : (rr < 4 ? id + size_t(3 * pj + rr - 1) * S : ih + size_t(9 * pj + rr - 4) * S);
             float* rowp2 = rr < 4 ? rowp : ih + size_t(9 * pj + rm - 4) * S;
-            point16_core<L, NORM, true>(x, y, z, r2, tb, rr, 10 * j, ir, rowp, rowp2, live);
+            point16_core<L, NORM, true>(x, y, z, r2, tb, rr, ir, rowp, rowp2, live);
         } else {
             float* rowp = slots + size_t(10 * pj + r) * S;
-            point16_core<L, NORM, false>(x, y, z, r2, tb, rr, 10 * j, ir, rowp, rowp, live);
+            point16_core<L, NORM, false>(x, y, z, r2, tb, rr, ir, rowp, rowp, live);
             if (bulk && live) {  // rows 16-byte aligned at both ends: one copy per global row
                 fence_proxy_async_smem();
                 const int64_t gp = p0 + pj;
