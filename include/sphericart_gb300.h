@@ -153,8 +153,8 @@ typedef enum {
  * 3 = 256 columns).
  * The POINT default (no shape given and none tuned) fills ~48 KB tiles (FP32,
  * bf16) or up to 32 points in <= 74 KB with one warp per block (FP64, bound by
- * the FP64 pipe), and with FP32 gradients from l_max 10 runs 4 lanes per
- * point on 8-point tiles, with FP32 Hessians 10 lanes per point where that
+ * the FP64 pipe), and with FP32 gradients from l_max 9 (normalized 8) runs 4
+ * lanes per point on 8-point tiles, with FP32 Hessians 10 lanes per point where that
  * measured faster (scaled l_max 7..16, normalized 6..15; ROW above); when a call
  * has fewer than 2 x SMs x
  * warps_per_block tiles, it runs fewer warps per block so that the blocks

@@ -285,9 +285,13 @@ size_t point4_row_bytes(int L, int elem) { return size_t(elem) * 4 * size_t(poin
 
 // Default shape of the 4-lanes-per-point tile: 8 points per warp (all 32
 // lanes), point4_default_warps warps per block, a grid of 16 blocks per SM
-// scheduled in waves (measured on GB300, 1M points, FP32 gradients).
+// scheduled in waves (measured on GB300, 1M points, FP32 gradients). Small
+// tiles take 8 warps (l_max 9: 6.68 against 6.23 TB/s). At l_max 16 a block of
+// 4 tiles fills an SM's shared memory alone, and 2-warp blocks keep 6 warps
+// resident instead of 4: 3.74 -> 5.79 TB/s (persistent; 5.51 in waves).
 sph_launch default_point4_fwd(int L, int elem) {
-    (void)elem;
+    if (L <= 9) return sph_launch{8, 8, 16, 4};
+    if (L >= 16 && elem == 4) return sph_launch{8, 2, 0, 4};
     return sph_launch{8, point4_default_warps(L), 16, 4};
 }
 
@@ -350,10 +354,12 @@ bool point10_default(int L, int hess, int normalized, int dtype, int out, int64_
 }
 
 // Whether the POINT default (no shape given, none tuned) runs 4 lanes per
-// point: FP32 arithmetic with gradients, no Hessians, l_max >= 10 (where the
-// one-lane tile that fits shared memory leaves most lanes idle).
-bool point4_default(int L, int grad, int elem, int hess, int hc) {
-    return grad && !hess && !hc && elem != 8 && L >= kPoint4MinL;
+// point: FP32 arithmetic with gradients, no Hessians, from l_max 9
+// (normalized 8), where the one-lane tile that fits shared memory leaves lanes
+// idle or leaves by plain stores.
+bool point4_default(int L, int grad, int elem, int hess, int hc, int normalized) {
+    return grad && !hess && !hc && elem != 8 && L >= point4_min_l_single(normalized) &&
+           (elem == 4 || L >= 9);  // bf16 at l_max 8: one lane 4.17, four 3.78 TB/s
 }
 
 sph_launch default_point_bwd(int L, int elem, int dbw) {
@@ -674,7 +680,7 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
         const int hess = ddsph ? 1 : 0;
         if (from_default && a.launch.points_per_tile == 0 && a.launch.warps_per_block == 0 &&
             a.launch.blocks_per_sm == 0 && a.launch.lanes_per_point == 0) {
-            if (point4_default(l_max, grad, eo, hess, hc))
+            if (point4_default(l_max, grad, eo, hess, hc, normalized))
                 a.launch.lanes_per_point = 4;
             else if (point10_default(l_max, hess, normalized, dtype, out, n))
                 a.launch.lanes_per_point = 10;
@@ -933,7 +939,7 @@ int sphericart_launch_info(int l_max, int dtype, int out, int grad, int hess, in
         }
         const bool none = s.points_per_tile == 0 && s.warps_per_block == 0 && s.blocks_per_sm == 0 &&
                           s.lanes_per_point == 0;
-        const bool four = s.lanes_per_point == 4 || (none && point4_default(l_max, grad, eo, hess, hc ? 1 : 0));
+        const bool four = s.lanes_per_point == 4 || (none && point4_default(l_max, grad, eo, hess, hc ? 1 : 0, 0));
         // (the scaled form's choice: launch_info takes no normalized flag)
         const bool ten = s.lanes_per_point == 10 || (none && !four && point10_default(l_max, hess, 0, dtype, out, 0));
         const bool sixteen = s.lanes_per_point == 16;

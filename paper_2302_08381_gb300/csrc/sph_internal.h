@@ -98,8 +98,13 @@ struct FwdArgs {
 };
 
 // Smallest l_max at which FP32 gradient tiles run 4 lanes per point (one per
-// output plane) by default, in single-set launches and in ragged batches.
+// output plane) by default, in ragged batches.
 constexpr int kPoint4MinL = 10;
+// ... and of single-set launches alone: the 8-warp 4-lane shape against the
+// one-lane default, 1M points: l_max 9 (even K: the one-lane tile leaves by
+// plain stores) 6.68 against 5.07 TB/s, normalized 6.65 against 4.11; l_max 8
+// normalized 6.56 against 5.97, scaled 6.63 against 6.55 (kept).
+SPH_HD constexpr int point4_min_l_single(int normalized) { return normalized ? 8 : 9; }
 
 // Shared-memory row stride (elements) of the 4-lanes-per-point POINT tile
 // and how the tile leaves shared memory:
