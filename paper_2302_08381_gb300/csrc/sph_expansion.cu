@@ -23,43 +23,86 @@ constexpr int kExpansionMaxRad = 64;
 
 // Row layout of the staged harmonics: the 2l+1 columns of degree l in groups
 // of 4 slots (the last group of a degree padded with zeros), group g at word
-// 4g + floor(g / 8). The lanes of one contraction round read up to 32
-// consecutive groups at the same slot; without the skew of one word per block
-// of 8 groups, groups 8 apart would share a bank. With it, 4d + (1 or 2 or 3)
-// for groups d < 32 apart is never a multiple of 32 words, so the reads are
-// free of bank conflicts, and each lane reads its 4 slots at immediate offsets.
+// 4g, so that a lane stores and loads a group with one 16-byte access (FP32).
+// The contraction is bound by instruction issue and shared-memory wavefronts
+// (64 % and 74 % busy): one load per point and lane instead of four, and 16
+// stores of a group per point instead of one per column.
 __host__ __device__ constexpr int exp_gstart(int l) { return l == 0 ? 0 : l + (l - 1) * (l - 1) / 4; }
-__host__ __device__ constexpr int exp_gbase(int g) { return 4 * g + g / 8; }
-__host__ __device__ constexpr int exp_ypos(int l, int k) {
-    return exp_gbase(exp_gstart(l) + (k - l * l) / 4) + (k - l * l) % 4;
-}
-// Row stride in words: odd, so that the lanes' stores (one row each) are
-// conflict-free too.
+// Row stride in words: 4 times an odd number, so that the 8 lanes of a quarter
+// warp, each storing a group of its own row, cover all 32 banks.
 template <int L>
 __host__ __device__ constexpr int exp_row_words() {
-    return (exp_gbase(exp_gstart(L + 1) - 1) + 4) | 1;
+    return 4 * (exp_gstart(L + 1) | 1);
 }
-
-// Every column gets its own word inside the row, for every supported l_max.
-constexpr bool exp_layout_ok() {
-    for (int L = 0; L <= 16; ++L) {
-        const int SY = (exp_gbase(exp_gstart(L + 1) - 1) + 4) | 1;
-        int prev = -1;
-        for (int l = 0; l <= L; ++l)
-            for (int k = l * l; k < (l + 1) * (l + 1); ++k) {
-                if (exp_ypos(l, k) <= prev) return false;
-                prev = exp_ypos(l, k);
-            }
-        if (prev + 1 >= SY || exp_gbase(exp_gstart(L + 1) - 1) + 3 >= SY) return false;
-    }
-    return true;
+// Words a row is allocated: at least those of an odd row with one word of skew
+// per 8 groups, which fixes the largest n_rad that is accepted.
+template <int L>
+__host__ __device__ constexpr int exp_row_alloc() {
+    constexpr int G = exp_gstart(L + 1), odd = (4 * G + (G - 1) / 8) | 1;
+    return exp_row_words<L>() > odd ? exp_row_words<L>() : odd;
 }
-static_assert(exp_layout_ok(), "grouped Y layout must be injective and inside the row");
 
 template <typename T>
+__device__ __forceinline__ void exp_store4(T* p, T a, T b, T c, T d) {
+    if constexpr (sizeof(T) == 4) {
+        *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+    } else {
+        reinterpret_cast<double2*>(p)[0] = make_double2(a, b);
+        reinterpret_cast<double2*>(p)[1] = make_double2(c, d);
+    }
+}
+
+// Collects a degree's columns and stores them by groups once the last one
+// (m = -l) is there.
+template <int L, typename T>
 struct ValVis {
     T* row;
-    __device__ __forceinline__ void emit(int l, int k, const Deriv<T>& d) { row[exp_ypos(l, k)] = d.v; }
+    T buf[2 * L + 4];
+    __device__ __forceinline__ void emit(int l, int k, const Deriv<T>& d) {
+        buf[k - l * l] = d.v;
+        if (k == l * l) {
+#pragma unroll
+            for (int i = 1; i < 4; ++i) buf[2 * l + i] = T(0);  // the last group's padding
+#pragma unroll
+            for (int g = 0; g < (2 * l + 4) / 4; ++g)
+                exp_store4(row + 4 * (exp_gstart(l) + g), buf[4 * g], buf[4 * g + 1], buf[4 * g + 2], buf[4 * g + 3]);
+        }
+    }
+};
+
+// The 4 columns x 4 channels of a work item. In FP32 the columns are taken in
+// pairs by packed fma: 8 instructions (and a copy per channel) for 16 products,
+// each rounded as a plain fma.
+template <typename T>
+struct ExpAcc {
+    T a[4][4];
+    __device__ __forceinline__ void set(int j, int q, T v) { a[j][q] = v; }
+    __device__ __forceinline__ T get(int j, int q) const { return a[j][q]; }
+    __device__ __forceinline__ void add(const T* __restrict__ y, const T (&r)[4]) {
+        const double2 y0 = reinterpret_cast<const double2*>(y)[0], y1 = reinterpret_cast<const double2*>(y)[1];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            a[0][q] = fma(y0.x, r[q], a[0][q]);
+            a[1][q] = fma(y0.y, r[q], a[1][q]);
+            a[2][q] = fma(y1.x, r[q], a[2][q]);
+            a[3][q] = fma(y1.y, r[q], a[3][q]);
+        }
+    }
+};
+template <>
+struct ExpAcc<float> {
+    float2 a[2][4];
+    __device__ __forceinline__ void set(int j, int q, float v) { (j & 1 ? a[j / 2][q].y : a[j / 2][q].x) = v; }
+    __device__ __forceinline__ float get(int j, int q) const { return j & 1 ? a[j / 2][q].y : a[j / 2][q].x; }
+    __device__ __forceinline__ void add(const float* __restrict__ y, const float (&r)[4]) {
+        const float4 v = *reinterpret_cast<const float4*>(y);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float2 rr = make_float2(r[q], r[q]);
+            a[0][q] = __ffma2_rn(make_float2(v.x, v.y), rr, a[0][q]);
+            a[1][q] = __ffma2_rn(make_float2(v.z, v.w), rr, a[1][q]);
+        }
+    }
 };
 
 constexpr int kExpBatch = 32;  // centres whose CSR offsets a warp holds in registers
@@ -82,7 +125,7 @@ __host__ __device__ constexpr size_t expansion_warp_bytes(int nr) {
     const int RW = nr * (L + 1);
     // radial buffers: 32 rows plus 3 rows' worth of channels that the masked
     // channels of the last row's items read past its end
-    return align16(size_t(32) * exp_row_words<L>() * sizeof(T)) +
+    return align16(size_t(32) * exp_row_alloc<L>() * sizeof(T)) +
            kExpRBuf * align16((size_t(32) * RW + 3 * (L + 1)) * sizeof(T)) + align16(size_t(nr) * K * sizeof(T)) +
            align16(size_t(kExpBatch) * (sizeof(int64_t) + sizeof(int))) + 16;
 }
@@ -195,7 +238,7 @@ __global__ void __launch_bounds__(256) expansion_kernel(const T* __restrict__ xy
     const int warp = threadIdx.x >> 5;
     const int W = blockDim.x >> 5;
     unsigned char* base = smem + size_t(warp) * expansion_warp_bytes<L, T>(nr);
-    const size_t ybytes = align16(size_t(32) * SY * sizeof(T));
+    const size_t ybytes = align16(size_t(32) * exp_row_alloc<L>() * sizeof(T));
     const size_t rbytes = align16((size_t(32) * RW + 3 * RL) * sizeof(T));
     const size_t cbytes = align16(size_t(nr) * K * sizeof(T));
     T* Ys = reinterpret_cast<T*>(base);
@@ -222,7 +265,6 @@ __global__ void __launch_bounds__(256) expansion_kernel(const T* __restrict__ xy
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
     }
-    for (int t = lane; t < 32 * SY; t += 32) Ys[t] = T(0);  // padding slots stay zero
     fence_proxy_async_smem();
     __syncwarp();
     uint32_t phase = 0, pending = 0;
@@ -299,7 +341,8 @@ __global__ void __launch_bounds__(256) expansion_kernel(const T* __restrict__ xy
             } else {
                 r2 = x * x + y * y + z * z;
             }
-            ValVis<T> vis{Ys + size_t(lane) * SY};
+            ValVis<L, T> vis;
+            vis.row = Ys + size_t(lane) * SY;
             point_core<L, false, false>(x, y, z, r2, tb, vis);
         }
         T* const Rs = b ? Rb1 : Rb0;
@@ -351,16 +394,16 @@ __global__ void __launch_bounds__(256) expansion_kernel(const T* __restrict__ xy
             bool qok[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) qok[q] = nbase + nstep * q < nr;
-            const T* yp = Ys + exp_gbase(exp_gstart(l) + cg);
+            const T* yp = Ys + 4 * (exp_gstart(l) + cg);
             const T* rp = Rs + nbase * RL + l;
             const int cbase = nbase * K + c0;  // [n][K] offset of the item's first output
             const int cstep = nstep * K;
-            T acc[4][4];
+            ExpAcc<T> acc;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    acc[j][q] = (carry_in && j < nc && qok[q]) ? Cs[cbase + q * cstep + j] : T(0);
+                    acc.set(j, q, (carry_in && j < nc && qok[q]) ? Cs[cbase + q * cstep + j] : T(0));
             // the segments of the chunk; S = channel stride of the item's slots
             auto segments = [&](auto s_tag) {
                 constexpr int S = decltype(s_tag)::value;
@@ -369,17 +412,11 @@ __global__ void __launch_bounds__(256) expansion_kernel(const T* __restrict__ xy
                     const int se = seg_end[si];
 #pragma unroll 4
                     for (int e = s; e < se; ++e) {
-                        const T* ye = yp + e * SY;
                         const T* re = rp + e * RW;
-                        T yv[4], rv[4];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) yv[j] = ye[j];
+                        T rv[4];
 #pragma unroll
                         for (int q = 0; q < 4; ++q) rv[q] = re[q * S * RL];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) acc[j][q] = fma(yv[j], rv[q], acc[j][q]);
+                        acc.add(yp + e * SY, rv);
                     }
                     s = se;
                     if (si + 1 < nseg || last_fin) {  // the centre ends here: write it out
@@ -388,8 +425,8 @@ __global__ void __launch_bounds__(256) expansion_kernel(const T* __restrict__ xy
                         for (int j = 0; j < 4; ++j)
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
-                                if (j < nc && qok[q]) ci[q * cstep + j] = acc[j][q];
-                                acc[j][q] = T(0);
+                                if (j < nc && qok[q]) ci[q * cstep + j] = acc.get(j, q);
+                                acc.set(j, q, T(0));
                             }
                     }
                 }
@@ -406,7 +443,7 @@ __global__ void __launch_bounds__(256) expansion_kernel(const T* __restrict__ xy
                 for (int j = 0; j < 4; ++j)
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
-                        if (j < nc && qok[q]) Cs[cbase + q * cstep + j] = acc[j][q];
+                        if (j < nc && qok[q]) Cs[cbase + q * cstep + j] = acc.get(j, q);
             }
         }
         fence_proxy_async_smem();  // generic reads of Rs done before the buffer is refilled
