@@ -45,7 +45,10 @@ def _check_points(xyz: torch.Tensor, name: str = "xyz") -> None:
 
 
 def _stream(device) -> int:
-    return torch.cuda.current_stream(device).cuda_stream
+    # the handle alone: 0.2 us, where building torch's Stream object takes 2
+    if device.index is None:
+        return torch.cuda.current_stream(device).cuda_stream
+    return torch._C._cuda_getCurrentRawStream(device.index)
 
 
 def _launch(launch):
