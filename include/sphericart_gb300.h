@@ -79,7 +79,9 @@ typedef enum { SPH_Q_NATIVE = 0, SPH_Q_F64 = 1 } sph_qprec;
 
 /* Kernel family. AUTO picks, by measurement on GB300: DEGREE for FP64
  * arithmetic without Hessians (the mixed mode; SPH_F64 from l_max 14, with
- * gradients from l_max 9); else
+ * gradients from l_max 9, and by the number of points from l_max 11, with
+ * gradients 5: launch_info, which takes none, reports the choice for few
+ * points); else
  * ROW for FP32 Hessians with FP32 storage up to l_max 63, from l_max 16
  * (below 8,192 points 14) in
  * the normalized form and beyond SPH_MAX_L_POINT in the scaled one
@@ -145,10 +147,10 @@ typedef enum {
  *                    SLICE: 8, 16 or 32 (0 = by l_max)
  * DEGREE kernels read warps_per_block (0..8, 0 = by shared memory),
  * blocks_per_sm and lanes_per_point (1, 2 or 4 lanes per point for DEGREE, 0 =
- * by measurement; DEGREE_DOWN takes 1). ROW kernels read warps_per_block
- * (forward 0..2, backward 0..8; 0 = one block of up to 12, backward 16, warps
- * per SM, 2 with Hessians),
- * blocks_per_sm, and lanes_per_point as the forward window policy (0 = by
+ * by measurement, for FP64 arithmetic also by the number of points, up to 8;
+ * launch_info reports the least; DEGREE_DOWN takes 1). ROW kernels read
+ * warps_per_block (forward 0..2, backward 0..8; 0 = one block of up to 12
+ * (backward 16) warps per SM, 2 with Hessians), blocks_per_sm, and lanes_per_point as the forward window policy (0 = by
  * l_max, 1, 2; with Hessians 0/2 = 136 columns, 1 = one degree of l_max,
  * 3 = 256 columns).
  * The POINT default (no shape given and none tuned) fills ~48 KB tiles (FP32,

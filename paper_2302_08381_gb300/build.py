@@ -49,7 +49,7 @@ def _units():
     for l in range(MAX_L_POINT + 1):
         units.append(("sph_point_inst.cu", f"point_L{l}.o", [f"-DSPH_INST_L={l}"]))
     units.append(("sph_degree.cu", "sph_degree_down.o", ["-DSPH_DEGREE_DOWN=1"]))
-    for lpp in (1, 2, 4):
+    for lpp in (1, 2, 4, 8):
         units.append(("sph_degree.cu", f"sph_degree_up{lpp}.o", ["-DSPH_DEGREE_DOWN=0", f"-DSPH_DEGREE_LPP={lpp}"]))
     for part in (0, 1):
         units.append(("sph_row.cu", f"sph_row_{part}.o", [f"-DSPH_ROW_PART={part}"]))

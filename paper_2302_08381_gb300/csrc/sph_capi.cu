@@ -107,23 +107,19 @@ const void* upload_packed(void*& slot, int dtype, Pack pack) {
 
 void* g_down32[kMaxDevices] = {nullptr};
 void* g_down64[kMaxDevices] = {nullptr};
+void* g_deg64[kMaxDevices] = {nullptr};
 
 }  // namespace
 
-const void* device_tables(int dtype) {
-    const int d = current_device();
-    if (d < 0) {
-        set_error("no current CUDA device");
-        return nullptr;
-    }
-    std::lock_guard<std::mutex> lk(g_mu);
-    void*& slot = (dtype == SPH_F64) ? g_tab64[d] : g_tab32[d];
+namespace {
+
+// (g_mu held) Packed per-(l, m) entries of kSliceTables values, see sph_internal.h:
+//   [0] a (m <= l-2), d_l (m = l-1), 0 (m = l)   [1] b (m <= l-2), else 0
+//   [2] Qtilde_l^l on the diagonal, else 0        [3] e
+//   [4] f   [5] g2   [6] g3   [7] g4
+const void* slice_tables(int d, int dtype) {
     const HostTables& h = host_tables();
-    // Packed per-(l, m) entries of kSliceTables values, see sph_internal.h:
-    //   [0] a (m <= l-2), d_l (m = l-1), 0 (m = l)   [1] b (m <= l-2), else 0
-    //   [2] Qtilde_l^l on the diagonal, else 0        [3] e
-    //   [4] f   [5] g2   [6] g3   [7] g4
-    return upload_packed(slot, dtype, [&](int l, int m, int i, double* v) {
+    return upload_packed(dtype == SPH_F64 ? g_tab64[d] : g_tab32[d], dtype, [&](int l, int m, int i, double* v) {
         v[0] = m <= l - 2 ? h.a[i] : (m == l - 1 ? h.d[i] : 0.0);
         v[1] = m <= l - 2 ? h.b[i] : 0.0;
         v[2] = m == l ? h.qll[i] : 0.0;
@@ -133,6 +129,39 @@ const void* device_tables(int dtype) {
         v[6] = h.g3[i];
         v[7] = h.g4[i];
     });
+}
+
+// (g_mu held) The tables of degree_f64_kernel.
+const void* degree_f64_tables(int d) {
+    const HostTables& h = host_tables();
+    static_assert(kF64Tables == kSliceTables, "upload_packed's entry size");
+    return upload_packed(g_deg64[d], SPH_F64, [&](int l, int m, int i, double* v) {
+        // 1 where the state it multiplies is zero: a product of normal numbers
+        v[0] = m <= l - 2 ? h.a[i] : (m == l - 1 ? h.d[i] : 1.0);
+        v[1] = m <= l - 2 ? h.b[i] : 1.0;
+        v[2] = m == l ? h.qll[i] : 0.0;
+        const double unfold = m == 0 ? 1.0 / h.inv_sqrt2 : 1.0;
+        v[3] = h.fz[i] * unfold;
+        v[4] = h.e[i] * unfold;
+        v[5] = v[6] = v[7] = 0.0;
+    });
+}
+
+}  // namespace
+
+// The first use of a precision's tables uploads all of them (the packed ones
+// and those of the DEGREE FP64 or ROW FP32 kernels), so that after any eager
+// call that needs tables every kernel of that precision can be captured.
+const void* device_tables(int dtype) {
+    const int d = current_device();
+    if (d < 0) {
+        set_error("no current CUDA device");
+        return nullptr;
+    }
+    if (dtype != SPH_F64 && !device_row_tables()) return nullptr;
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (dtype == SPH_F64 && !degree_f64_tables(d)) return nullptr;
+    return slice_tables(d, dtype);
 }
 
 const void* device_tables_down(int dtype) {
@@ -155,6 +184,16 @@ const void* device_tables_down(int dtype) {
     });
 }
 
+const void* device_tables_f64() {
+    return device_tables(SPH_F64) ? g_deg64[current_device()] : nullptr;
+}
+
+bool device_tables_f64_ready() {
+    const int d = current_device();
+    std::lock_guard<std::mutex> lk(g_mu);
+    return d >= 0 && g_deg64[d] != nullptr;
+}
+
 // Coefficient streams of the ROW kernels (FP32): entry (d * 8 + k) * 8 + j
 // holds, for degree d and channel m = j + 8k (lane j, slot k), the float4
 // {A, B, S, e} of the packed tables and, in a second array after the first,
@@ -169,6 +208,7 @@ const void* device_row_tables() {
     static void* slots[kMaxDevices] = {nullptr};
     std::lock_guard<std::mutex> lk(g_mu);
     if (slots[d]) return slots[d];
+    if (!slice_tables(d, SPH_F32)) return nullptr;
     const HostTables& h = host_tables();
     constexpr int kEntries = kRowLanes * kRowDegrees * kRowSlots;
     std::vector<float> host(size_t(kEntries) * 9, 0.f);
@@ -478,14 +518,29 @@ bool valid_lanes(const sph_launch& s) {
 
 bool aligned(const void* p, size_t a) { return reinterpret_cast<uintptr_t>(p) % a == 0; }
 
-// Lanes per point of the upward DEGREE kernel when the caller leaves it 0
-// (measured on GB300: FP64 prefers 1 lane per point below l_max 10, 2 up to
-// l_max ~ 24 and 4 above, FP32 arithmetic with FP64 Q ("mixed") 2, FP32 /
-// bf16 storage 4).
+// Lanes per point of the upward DEGREE kernel when the caller leaves it 0:
+// FP32 arithmetic 4; FP64 arithmetic at least these, see degree_f64_lpp.
 int degree_default_lpp(int l_max, int dtype, int qprec) {
     if (dtype == SPH_F64) return l_max >= 24 ? 4 : (l_max >= 10 ? 2 : 1);
     if (qprec == SPH_Q_F64) return 2;
     return 4;
+}
+
+// FP64 arithmetic (degree_f64_kernel). A point's lane-private state grows with
+// l_max, and with few warps on an SM the latency of the integer products shows:
+// more lanes per point are more warps, until the lanes with m > l cost more.
+// Measured on GB300, normalized, ms at 2 / 4 / 8 lanes: gradients, 300k points
+// l_max 8 .65/.74/-; 200k l_max 12 .87/.85/-, 20 2.57/1.97/-, 30 6.3/4.3/3.9; 100k
+// l_max 50 12.6/7.4/5.4; values, 200k l_max 12 .23/.25/-, 20 .60/.55/-, 30
+// 1.7/1.1/-; 100k l_max 40 1.9/1.15/-, 50 2.7/2.0/1.6. Few points: enough lanes
+// for about six warps per SM (10k points, gradients, l_max 20 at 2 / 4 / 8 lanes:
+// 181/134/167 us; 1k points 248/97/72 us).
+int degree_f64_lpp(int64_t n, int l_max, bool grad, bool mixed) {
+    int lpp;
+    if (grad) lpp = l_max > 26 ? 8 : (l_max >= (mixed ? 16 : 12) ? 4 : 2);
+    else lpp = l_max > 44 ? 8 : (l_max >= 20 ? 4 : 2);
+    while (lpp < 8 && n * lpp < int64_t(6) * 32 * sm_count()) lpp *= 2;
+    return lpp;
 }
 
 }  // namespace
@@ -499,6 +554,17 @@ bool point_hybrid_wins(int l_max, int dtype, bool grad) {
 }
 
 namespace {
+
+// FP64 requests below auto_family's DEGREE limits that run faster there all
+// the same, by the number of points. Measured on GB300 (us, POINT / DEGREE):
+// gradients, normalized (scaled), 400k points l_max 6 601 / 531 (365 / 440), 7
+// 1172 / 623 (703 / 525); 300k l_max 8 1195 / 639 (697 / 496); 1k points l_max 4
+// 19 / 17, 5..8 33..52 / 21..27; values, 200k points l_max 12 248 / 224; 50k
+// l_max 10 52 / 62; 10k l_max 12 29 / 31.
+bool f64_prefers_degree(int64_t n, int l_max, bool grad) {
+    if (grad) return n >= 256 && (l_max >= 7 || (l_max >= 5 && n <= 8192));
+    return n >= 32768 && l_max >= 11;
+}
 
 // AUTO kernel family of a forward request (measured on GB300). POINT
 // (compile-time l_max, TMA bulk stores) wins whenever it applies in FP32, and
@@ -622,6 +688,16 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
     const bool hess_bf16 = ddsph && out == SPH_OUT_BF16;
     if (fam == SPH_KERNEL_AUTO)
         fam = auto_family(l_max, dtype, out, qprec, ddsph != nullptr, dsph != nullptr, normalized, n);
+    if (kernel == SPH_KERNEL_AUTO && !launch && dtype == SPH_F64 && !ddsph && f64_prefers_degree(n, l_max, grad)) {
+        // POINT needs no device tables: a call captured before any upload stays there
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (device_tables_f64_ready() ||
+            (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) == cudaSuccess &&
+             cap == cudaStreamCaptureStatusNone))
+            fam = SPH_KERNEL_DEGREE;
+        else
+            cudaGetLastError();
+    }
     int hc = 0;
     if (fam == SPH_KERNEL_POINT_HC) {
         if (l_max > kHcMaxL || ddsph || mixed || out != SPH_OUT_SAME) {
@@ -740,7 +816,7 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
             set_error("DEGREE launch: warps_per_block must be in [0,8] and blocks_per_sm in [0,32]");
             return SPH_EINVAL;
         }
-        const int lpp = a.launch.lanes_per_point;
+        int lpp = a.launch.lanes_per_point;
         if (lpp != 0 && lpp != 1 && lpp != 2 && lpp != 4) {
             set_error("DEGREE launch: lanes_per_point must be 0, 1, 2 or 4");
             return SPH_EINVAL;
@@ -749,18 +825,17 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
             set_error("DEGREE_DOWN runs one lane per point (the downward recursion is sequential in m)");
             return SPH_EINVAL;
         }
+        if (lpp == 0)
+            lpp = dtype == SPH_F64 || mixed ? degree_f64_lpp(n, l_max, grad, mixed)
+                                            : degree_default_lpp(l_max, dtype, qprec);
         int e;
         if (fam == SPH_KERNEL_DEGREE_DOWN)
             e = degree_fwd_down(a);
-        else if (lpp == 1)
-            e = degree_fwd_up1(a);
-        else if (lpp == 4)
-            e = degree_fwd_up4(a);
-        else if (lpp == 2)
-            e = degree_fwd_up2(a);
         else
-            e = degree_default_lpp(l_max, dtype, qprec) == 1 ? degree_fwd_up1(a)
-                : degree_default_lpp(l_max, dtype, qprec) == 4 ? degree_fwd_up4(a) : degree_fwd_up2(a);
+            e = lpp == 1   ? degree_fwd_up1(a)
+                : lpp == 2 ? degree_fwd_up2(a)
+                : lpp == 4 ? degree_fwd_up4(a)
+                           : degree_fwd_up8(a);
         if (e == int(cudaErrorInvalidConfiguration)) {
             set_error("DEGREE launch shape needs more shared memory per block than the device allows");
             return SPH_EINVAL;

@@ -41,6 +41,7 @@
 
 #include "sph_core.cuh"
 #include "sph_internal.h"
+#include "sph_mul64.cuh"
 
 #ifndef SPH_DEGREE_DOWN
 #define SPH_DEGREE_DOWN 0
@@ -96,9 +97,9 @@ struct DegTab<float, true> {
     __device__ __forceinline__ float f(int i) const { return c_tabf[i]; }
 };
 
-template <int LPP, typename TO, bool GRAD>
+template <int LPP, typename TO, bool GRAD, int ST = kSt>
 __host__ __device__ constexpr size_t degree_stage_bytes() {
-    return deg_align(size_t(GRAD ? 4 : 1) * (32 / LPP) * kSt * sizeof(TO));
+    return deg_align(size_t(GRAD ? 4 : 1) * (32 / LPP) * ST * sizeof(TO));
 }
 
 // Number of state columns (each one entry per point of the warp) a warp keeps.
@@ -260,30 +261,30 @@ __device__ __forceinline__ void down_chunk(int l, int m_lo, int m_hi, int sp0, i
 
 // Stores `np` rows of the staged columns: lane t < ncols owns global column
 // colA0 + t (t < nA) or offB + t (t >= nA) of every point in the tile.
-template <int PPW, typename TO>
+template <int PPW, int ST = kSt, typename TO>
 __device__ __forceinline__ void store_rows(TO* __restrict__ g, int64_t rstride, const TO* __restrict__ s, int np) {
     if (np == PPW) {
 #pragma unroll 8
-        for (int p = 0; p < PPW; ++p) g[p * rstride] = s[p * kSt];
+        for (int p = 0; p < PPW; ++p) g[p * rstride] = s[p * ST];
     } else {
-        for (int p = 0; p < np; ++p) g[p * rstride] = s[p * kSt];
+        for (int p = 0; p < np; ++p) g[p * rstride] = s[p * ST];
     }
 }
 
-template <int PPW, bool GRAD, typename TO>
+template <int PPW, bool GRAD, int ST = kSt, typename TO>
 __device__ __forceinline__ void flush_stage(const TO* __restrict__ stw, TO* __restrict__ sph_t,
                                             TO* __restrict__ dsph_t, int64_t K, int np, int ncols, int nA,
                                             int64_t colA0, int64_t offB, int lane) {
-    constexpr int PL = PPW * kSt;
+    constexpr int PL = PPW * ST;
     __syncwarp();
     if (lane < ncols) {
         const int64_t col = lane < nA ? colA0 + lane : offB + lane;
         const TO* s = stw + lane;
-        store_rows<PPW>(sph_t + col, K, s, np);
+        store_rows<PPW, ST>(sph_t + col, K, s, np);
         if (GRAD) {
-            store_rows<PPW>(dsph_t + col, 3 * K, s + PL, np);
-            store_rows<PPW>(dsph_t + K + col, 3 * K, s + 2 * PL, np);
-            store_rows<PPW>(dsph_t + 2 * K + col, 3 * K, s + 3 * PL, np);
+            store_rows<PPW, ST>(dsph_t + col, 3 * K, s + PL, np);
+            store_rows<PPW, ST>(dsph_t + K + col, 3 * K, s + 2 * PL, np);
+            store_rows<PPW, ST>(dsph_t + 2 * K + col, 3 * K, s + 3 * PL, np);
         }
     }
     __syncwarp();
@@ -434,6 +435,284 @@ __global__ void __launch_bounds__(256) degree_fwd_kernel(const TI* __restrict__ 
     }
 }
 
+#if !SPH_DEGREE_DOWN
+// --------------------------- FP64 arithmetic, upward in l (degree_f64_kernel)
+// GB300 issues one FP64 warp instruction per SM every 20 clocks, so the number
+// of FP64 instructions bounds this path. Two things cut it from 39 per pair of
+// columns (l, +-m) with normalized gradients to 11:
+//  * the derivatives of Eq. iter-deri are put together on the Q side first,
+//      dY/dx = X c_m + Q m c_{m-1},  X = x e Q_{l-1}^{m+1} - l u_x Q    (Y, Z likewise),
+//    with 1/r and m folded into the kept c_m and c_{m-1}: 9 fma and 12
+//    products (scaled: 6 and 12; values: 2 and 4);
+//  * ten of those products (values: all four) run on the integer pipe, whose
+//    issue slots idle beside the FP64 pipe (sph_mul64.cuh).
+// 200k points, l_max 30, normalized, values and gradients: 9.03 -> 3.92 ms (FP64
+// pipe about 60 % busy, issue 50 %). Linear maps from the columns of degree l - 1
+// take one FP64 instruction less, and were 2 % faster, but carry the larger
+// rounding of the m = 0 column into the gradients next to the poles (rms error
+// 7.9e-15 against 4.5e-15): not kept.
+// A lane owns the channels m = h (mod LPP) of its point. Their state (q1, q2)
+// and c_m, s_m, c_m / r, s_m / r, m c_{m-1} / r, m s_{m-1} / r (computed once per
+// point) is lane-private in shared memory, [slot][lane] pairs of doubles;
+// Q_{l-1}^{m+1} comes from the neighbouring lane by a shuffle. m = 0 is the same
+// code: c_0 = 1/sqrt2, s_0 = 0, against multipliers without the 1/sqrt2.
+// m values per chunk. Four planes of FP64 columns take half of the FP32 kernels'
+// chunk: the smaller stage leaves more warps on an SM (200k points, l_max 30: 3.97
+// against 4.05 ms, 300k, 8: 0.65 against 0.71); FP32 outputs and values alone are
+// 4..12 % faster with whole chunks.
+template <typename TO, bool GRAD>
+constexpr int kMC64 = GRAD && sizeof(TO) == 8 ? kMC / 2 : kMC;
+
+struct F64Point {
+    double x, y;
+    Mul64 z, r2;
+};
+
+// Lane-private pairs per slot: {q1, q2}, {c_m, s_m}, with gradients {m c_{m-1},
+// m s_{m-1}} and, normalized, {c_m, s_m} / r.
+template <bool GRAD, bool NORM>
+__host__ __device__ constexpr int f64_pairs() { return GRAD ? (NORM ? 4 : 3) : 2; }
+__host__ __device__ constexpr int f64_slots(int L, int lpp) { return L / lpp + 2; }  // + 1: read ahead, zero
+
+template <int LPP, typename TO, bool GRAD, bool NORM>
+__host__ __device__ constexpr size_t f64_warp_bytes(int L) {
+    return degree_stage_bytes<LPP, TO, GRAD, 2 * kMC64<TO, GRAD> + 1>() + size_t(f64_pairs<GRAD, NORM>()) * f64_slots(L, LPP) * 32 * sizeof(double2);
+}
+
+// One step of one channel: everything that is computed from the state.
+struct F64Step {
+    double q;                       // Qtilde_l^m
+    double vc, vs;                  // Y^{+m}, Y^{-m}
+    double xc, xs, yc, ys, zc, zs;  // gradient planes of both columns
+};
+
+// FAST: the products that are not part of an fma on the integer pipe; returns
+// false where one of them has an operand out of its range (the caller then
+// repeats the step without FAST). A product with a factor that is zero by its
+// place (s_0, Q_{l-1}^{m+1} beyond the degree) is no such case: it is set to
+// zero. t: {A, B, S, f}, e; q: {Qtilde_{l-1}^m, Qtilde_{l-2}^m}; qr:
+// Qtilde_{l-1}^{m+1}; c, ci, c1: {c_m, s_m}, the same / r, m {c_{m-1}, s_{m-1}} / r.
+template <bool FAST, bool GRAD, bool NORM>
+__device__ __forceinline__ bool f64_step(int l, int m, const double4_32a& t, double e, const F64Point& P, double lx,
+                                         double ly, double lz, const double2& q, double qr, const double2& c,
+                                         const double2& ci, const double2& c1, F64Step& o) {
+    bool in = true;
+    // a * b, or 0 where it is not `used`
+    auto mul = [&](double a, const Mul64& b, bool used) {
+        if (!FAST) return used ? a * b.v : 0.0;
+        bool ok = b.ok;
+        const double p = b.fast(a, ok);
+        in = in && (ok || !used);
+        return used ? p : 0.0;
+    };
+    const bool m1 = m > 0;
+    // explicit fma: the same rounding in every variant (values-only or not)
+    // With gradients A z and B r2 stay on the FP64 pipe: with 12 products on the
+    // integer pipe its issue slots become the bound (l_max 30, 200k points: 4.2 ms;
+    // 3.9 so). Values have only these and two more (l_max 30: 1.10 against 1.40 ms).
+    const double az = GRAD ? t.x * P.z.v : mul(t.x, P.z, true), br = GRAD ? t.y * P.r2.v : mul(t.y, P.r2, true);
+    o.q = fma(az, q.x, fma(-br, q.y, t.z));
+    const Mul64 Q(o.q);
+    o.vc = mul(c.x, Q, true);
+    o.vs = mul(c.y, Q, m1);
+    if (GRAD) {
+        const double E1 = mul(qr, Mul64(e), m < l - 1);  // e Qtilde_{l-1}^{m+1}
+        const Mul64 E(E1);
+        double X = mul(P.x, E, m < l - 1), Y = mul(P.y, E, m < l - 1), Z = mul(q.x, Mul64(t.w), m < l);
+        if (NORM) {
+            X = fma(-lx, o.q, X);
+            Y = fma(-ly, o.q, Y);
+            Z = fma(-lz, o.q, Z);
+        }
+        const double tc = mul(c1.x, Q, m1), ts = mul(c1.y, Q, m > 1);
+        o.xc = fma(X, ci.x, tc);
+        o.xs = fma(X, ci.y, ts);
+        o.yc = fma(Y, ci.x, -ts);
+        o.ys = fma(Y, ci.y, tc);
+        const Mul64 Zm(Z);
+        const bool zu = NORM ? l > 0 : m < l;
+        o.zc = mul(ci.x, Zm, zu);
+        o.zs = mul(ci.y, Zm, zu && m1);
+    }
+    return in;
+}
+
+// Stages a step's columns (lanes that are `on`). FAST (FP32 and bfloat16
+// outputs): conversions on the integer pipe, false where one is out of their
+// range. For m = 0 both columns are the same slot, the second store wins.
+template <bool FAST, int PL, bool GRAD, typename TO>
+__device__ __forceinline__ bool f64_put(TO* __restrict__ st, int sp, int sm, const F64Step& o, bool on) {
+    bool in = true;
+    auto put = [&](int at, double v) {
+        TO r;
+        if constexpr (FAST) r = OutConv<TO>::cv(f32_of_f64(v, in));
+        else r = OutConv<TO>::cv(v);
+        if (on) st[at] = r;
+    };
+    put(sm, o.vs);
+    put(sp, o.vc);
+    if (GRAD) {
+        put(PL + sm, o.xs);
+        put(PL + sp, o.xc);
+        put(2 * PL + sm, o.ys);
+        put(2 * PL + sp, o.yc);
+        put(3 * PL + sm, o.zs);
+        put(3 * PL + sp, o.zc);
+    }
+    return in;
+}
+
+// The channels m_lo..m_hi of degree l (m_lo a multiple of
+// the chunk width): steps of LPP
+// channels, the same number in every lane of the warp; lanes with m > l only
+// take part in the shuffle. `st64`: this lane's state, pair i of slot k at
+// [32 (i NS + k)]; `qc` carries {q1, q2} of the lane's current channel.
+template <int LPP, bool GRAD, bool NORM, typename TO>
+__device__ __forceinline__ void f64_chunk(int l, int m_lo, int m_hi, int h, int lane, int sp0, int sm0,
+                                          const double* __restrict__ tab, const F64Point& P, double lx, double ly,
+                                          double lz, double2* __restrict__ st64, int NS, TO* __restrict__ st,
+                                          double2& qc) {
+    constexpr int PL = (32 / LPP) * (2 * kMC64<TO, GRAD> + 1);
+    constexpr unsigned kAll = 0xffffffffu;
+    const int up = (lane & ~(LPP - 1)) | ((h + 1) & (LPP - 1));  // the lane of channel m + 1
+    const double* const row = tab + size_t(kF64Tables) * tri(l, 0);
+    const int k0 = m_lo / LPP, steps = (m_hi - m_lo) / LPP + 1;
+#pragma unroll 1
+    for (int t = 0; t < steps; ++t) {
+        const int m = m_lo + LPP * t + h;
+        const int k = k0 + t;
+        const bool on = m <= l;
+        const double* en = row + kF64Tables * min(m, l);
+        const double4_32a t0 = *reinterpret_cast<const double4_32a*>(en);  // {A, B, S, f}
+        const double2 qn = st64[32 * (k + 1)];                             // the lane's next channel
+        const double2 c = st64[32 * (NS + k)];
+        double2 c1 = make_double2(0.0, 0.0), ci = c;
+        double e = 0.0, qr = 0.0;
+        if (GRAD) {
+            e = en[4];
+            c1 = st64[32 * (2 * NS + k)];
+            if (NORM) ci = st64[32 * (3 * NS + k)];
+            qr = qn.x;  // Qtilde_{l-1}^{m+1}
+            if (LPP > 1) qr = __shfl_sync(kAll, h == 0 ? qn.x : qc.x, up);
+        }
+        F64Step o;
+        const bool in = f64_step<true, GRAD, NORM>(l, m, t0, e, P, lx, ly, lz, qc, qr, c, ci, c1, o);
+        if (__any_sync(kAll, on && !in)) f64_step<false, GRAD, NORM>(l, m, t0, e, P, lx, ly, lz, qc, qr, c, ci, c1, o);
+        if (on) st64[32 * k] = make_double2(o.q, qc.x);
+        if (sizeof(TO) == 8) {
+            f64_put<false, PL, GRAD>(st, sp0 + m, sm0 - m, o, on);
+        } else if (__any_sync(kAll, on && !f64_put<true, PL, GRAD>(st, sp0 + m, sm0 - m, o, on))) {
+            f64_put<false, PL, GRAD>(st, sp0 + m, sm0 - m, o, on);
+        }
+        qc = qn;
+    }
+}
+
+template <typename TI, typename TO, bool GRAD, bool NORM, int LPP>
+__global__ void __launch_bounds__(256, 2) degree_f64_kernel(const TI* __restrict__ xyz, int64_t n, int L,
+                                                                           const double* __restrict__ tab,
+                                                                           double inv_sqrt2, TO* __restrict__ sph,
+                                                                           TO* __restrict__ dsph) {
+    constexpr int PPW = 32 / LPP;  // points per warp tile
+    constexpr int MC = kMC64<TO, GRAD>, ST = 2 * MC + 1;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const int W = blockDim.x >> 5;
+    const int pt = lane / LPP;
+    const int h = lane % LPP;
+    const int NS = f64_slots(L, LPP);
+    unsigned char* wbase = smem + size_t(warp) * f64_warp_bytes<LPP, TO, GRAD, NORM>(L);
+    TO* const stw = reinterpret_cast<TO*>(wbase);
+    TO* const stl = stw + pt * ST;
+    double2* const st64 = reinterpret_cast<double2*>(wbase + degree_stage_bytes<LPP, TO, GRAD, 2 * kMC64<TO, GRAD> + 1>()) + lane;
+    const int64_t K = int64_t(L + 1) * (L + 1);
+    const int64_t ntiles = (n + PPW - 1) / PPW;
+
+    for (int64_t tile = int64_t(blockIdx.x) * W + warp; tile < ntiles; tile += int64_t(gridDim.x) * W) {
+        const int64_t p0 = tile * PPW;
+        const int np = int(min(int64_t(PPW), n - p0));
+        double x = 0.0, y = 0.0, z = 0.0, ir = 1.0;
+        if (pt < np) {
+            x = double(xyz[3 * (p0 + pt)]);
+            y = double(xyz[3 * (p0 + pt) + 1]);
+            z = double(xyz[3 * (p0 + pt) + 2]);
+        }
+        if (NORM) {  // u = xyz / r, r2 = |u|^2 of the rounded u (0 at r = 0), as in unit_point
+            const double rr = fma(x, x, fma(y, y, z * z));
+            ir = rr > 0.0 ? 1.0 / sqrt(rr) : 0.0;
+            x *= ir;
+            y *= ir;
+            z *= ir;
+        }
+        const F64Point P{x, y, Mul64(z), Mul64(fma(z, z, fma(x, x, y * y)))};
+        TO* const sph_t = sph + p0 * K;
+        TO* const dsph_t = GRAD ? dsph + p0 * 3 * K : nullptr;
+
+        {  // (x + i y)^m of this lane's channels (Eq. iter-sc), steps of (x + i y)^LPP; the recursion state zeroed
+            const CS<double> xy{x, y};
+            CS<double> a{1.0, 0.0}, b{1.0, 0.0}, w{1.0, 0.0};  // ^m, ^(m-1) (h = 0: ^(m+LPP-1))
+#pragma unroll
+            for (int t = 0; t < LPP; ++t) {
+                if (t < h) a = a.times(xy);
+                if (t < (h > 0 ? h - 1 : LPP - 1)) b = b.times(xy);
+                w = w.times(xy);
+            }
+            for (int k = 0; k < NS; ++k) {
+                const bool m0 = k == 0 && h == 0;
+                const double2 c = make_double2(m0 ? inv_sqrt2 : a.c, a.s);
+                st64[32 * k] = make_double2(0.0, 0.0);
+                st64[32 * (NS + k)] = c;
+                if (GRAD) {
+                    const double f = m0 ? 0.0 : double(h + LPP * k) * ir;
+                    st64[32 * (2 * NS + k)] = make_double2(f * b.c, f * b.s);
+                    if (NORM) st64[32 * (3 * NS + k)] = make_double2(c.x * ir, c.y * ir);
+                    if (!m0) b = b.times(w);
+                }
+                a = a.times(w);
+            }
+        }
+
+        int l = 0;
+        while (l <= L) {
+            if (2 * l + 1 <= 2 * MC) {
+                // Whole small degrees la..lb, contiguous columns la^2 .. (lb+1)^2-1.
+                const int la = l;
+                int lb = l;
+                while (lb < L && (lb + 2) * (lb + 2) - la * la <= 2 * MC) ++lb;
+                const int colA0 = la * la;
+                for (int d = la; d <= lb; ++d) {
+                    const int c0 = d * d + d - colA0;
+                    const double dl = double(d);
+                    double2 qc = st64[0];
+                    f64_chunk<LPP, GRAD, NORM>(d, 0, d, h, lane, c0, c0, tab, P, dl * x, dl * y, dl * z, st64, NS, stl,
+                                               qc);
+                }
+                const int nc = (lb + 1) * (lb + 1) - colA0;
+                flush_stage<PPW, GRAD, ST>(stw, sph_t, dsph_t, K, np, nc, nc, colA0, colA0, lane);
+                l = lb + 1;
+            } else {
+                const int ctr = l * l + l;
+                const double dl = double(l);
+                const double lx = dl * x, ly = dl * y, lz = dl * z;
+                double2 qc = st64[0];
+                for (int m_lo = 0; m_lo <= l; m_lo += MC) {
+                    const int m_hi = min(l, m_lo + MC - 1);
+                    const int colA0 = ctr - m_hi;
+                    const int nA = m_lo == 0 ? 2 * m_hi + 1 : m_hi - m_lo + 1;
+                    const int nc = m_lo == 0 ? nA : 2 * nA;
+                    const int offB = m_lo == 0 ? colA0 : ctr + m_lo - nA;
+                    f64_chunk<LPP, GRAD, NORM>(l, m_lo, m_hi, h, lane, ctr - offB, ctr - colA0, tab, P, lx, ly, lz,
+                                               st64, NS, stl, qc);
+                    flush_stage<PPW, GRAD, ST>(stw, sph_t, dsph_t, K, np, nc, nA, colA0, offB, lane);
+                }
+                ++l;
+            }
+        }
+    }
+}
+#endif
+
 // Warps per block: enough to fill the SM in few blocks without one block
 // holding most of its shared memory.
 int default_warps(size_t per_warp) {
@@ -442,7 +721,7 @@ int default_warps(size_t per_warp) {
 }
 
 constexpr int kLPP = SPH_DEGREE_DOWN ? 1 : SPH_DEGREE_LPP;
-static_assert(kLPP == 1 || kLPP == 2 || kLPP == 4, "lanes per point: 1, 2 or 4");
+static_assert(kLPP == 1 || kLPP == 2 || kLPP == 4 || kLPP == 8, "lanes per point: 1, 2, 4 or 8 (FP64)");
 
 template <typename TI, typename TQ, typename TO, bool GRAD, bool NORM, bool DOWN, bool CT>
 int launch_degree(const FwdArgs& a, const TQ* tb) {
@@ -476,6 +755,58 @@ int launch_degree(const FwdArgs& a, const TQ* tb) {
         static_cast<TO*>(a.dsph));
     return int(cudaGetLastError());
 }
+
+#if !SPH_DEGREE_DOWN
+// The lane-private state of degree_f64_kernel takes more shared memory than
+// degree_fwd_kernel's columns: a block of the requested warps that does not
+// fit runs fewer, and one lane per point at l_max 128 runs two. What is
+// refused is decided by the size of degree_fwd_kernel's block, as for FP32.
+template <typename TI, typename TO, bool GRAD, bool NORM>
+int launch_f64(const FwdArgs& a, const double* tb) {
+    constexpr int PPW = 32 / kLPP;
+    auto kern = degree_f64_kernel<TI, TO, GRAD, NORM, kLPP>;
+    const size_t optin = size_t(max_smem_optin());
+    const size_t per_warp = f64_warp_bytes<kLPP, TO, GRAD, NORM>(a.l_max);
+    if (a.launch.warps_per_block > 0 &&
+        size_t(a.launch.warps_per_block) * degree_warp_bytes<kLPP, double, TO, GRAD, false>(a.l_max) > optin)
+        return int(cudaErrorInvalidConfiguration);
+    if (kLPP == 1 && per_warp > optin) return degree_fwd_up2(a);
+    int W = a.launch.warps_per_block > 0 ? a.launch.warps_per_block : default_warps(per_warp);
+    W = int(std::min<size_t>(W, optin / per_warp));
+    const size_t smem = size_t(W) * per_warp;
+    if (smem > 48 * 1024) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(reinterpret_cast<const void*>(kern), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(smem));
+        if (e != cudaSuccess) return int(e);
+    }
+    int bps = a.launch.blocks_per_sm;
+    if (bps <= 0) {
+        int occ = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, reinterpret_cast<const void*>(kern), 32 * W, smem) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            occ = 1;
+        }
+        bps = std::max(occ, 1);
+    }
+    const int64_t ntiles = (a.n + PPW - 1) / PPW;
+    const int64_t want = (ntiles + W - 1) / W;
+    const int grid = int(std::max<int64_t>(1, std::min<int64_t>(want, int64_t(bps) * sm_count())));
+    kern<<<grid, 32 * W, smem, static_cast<cudaStream_t>(a.stream)>>>(
+        static_cast<const TI*>(a.xyz), a.n, a.l_max, tb, host_tables().inv_sqrt2, static_cast<TO*>(a.sph),
+        static_cast<TO*>(a.dsph));
+    return int(cudaGetLastError());
+}
+
+template <typename TI, typename TO>
+int launch_f64_flags(const FwdArgs& a) {
+    const double* tb = static_cast<const double*>(device_tables_f64());
+    if (!tb) return int(cudaErrorMemoryAllocation);
+    if (a.dsph) return a.normalized ? launch_f64<TI, TO, true, true>(a, tb) : launch_f64<TI, TO, true, false>(a, tb);
+    return a.normalized ? launch_f64<TI, TO, false, true>(a, tb) : launch_f64<TI, TO, false, false>(a, tb);
+}
+#endif
 
 template <typename TI, typename TQ, typename TO, bool DOWN, bool CT>
 int launch_degree_flags(const FwdArgs& a, const TQ* tb) {
@@ -528,17 +859,22 @@ bool ensure_const_tables() {
 
 template <bool DOWN>
 int degree_fwd_dir(const FwdArgs& a) {
-    const int tdt = (a.dtype == SPH_F64 || a.qprec == SPH_Q_F64) ? SPH_F64 : SPH_F32;
-    const void* tb = DOWN ? device_tables_down(tdt) : device_tables(tdt);
-    if (!tb) return int(cudaErrorMemoryAllocation);
-    if (a.dtype == SPH_F64)
-        return launch_degree_flags<double, double, double, DOWN, false>(a, static_cast<const double*>(tb));
-    if (a.qprec == SPH_Q_F64) {
-        if (a.out == SPH_OUT_BF16)
-            return launch_degree_flags<float, double, __nv_bfloat16, DOWN, false>(a, static_cast<const double*>(tb));
-        return launch_degree_flags<float, double, float, DOWN, false>(a, static_cast<const double*>(tb));
+    if (a.dtype == SPH_F64 || a.qprec == SPH_Q_F64) {
+#if SPH_DEGREE_DOWN
+        const double* td = static_cast<const double*>(device_tables_down(SPH_F64));
+        if (!td) return int(cudaErrorMemoryAllocation);
+        if (a.dtype == SPH_F64) return launch_degree_flags<double, double, double, DOWN, false>(a, td);
+        if (a.out == SPH_OUT_BF16) return launch_degree_flags<float, double, __nv_bfloat16, DOWN, false>(a, td);
+        return launch_degree_flags<float, double, float, DOWN, false>(a, td);
+#else
+        if (a.dtype == SPH_F64) return launch_f64_flags<double, double>(a);
+        if (a.out == SPH_OUT_BF16) return launch_f64_flags<float, __nv_bfloat16>(a);
+        return launch_f64_flags<float, float>(a);
+#endif
     }
-    const float* tf = static_cast<const float*>(tb);
+#if SPH_DEGREE_LPP != 8
+    const float* tf = static_cast<const float*>(DOWN ? device_tables_down(SPH_F32) : device_tables(SPH_F32));
+    if (!tf) return int(cudaErrorMemoryAllocation);
     if (a.l_max <= kConstL) {
         if (!ensure_const_tables<DOWN>()) return int(cudaErrorMemoryAllocation);
         if (a.out == SPH_OUT_BF16) return launch_degree_flags<float, float, __nv_bfloat16, DOWN, true>(a, tf);
@@ -546,6 +882,9 @@ int degree_fwd_dir(const FwdArgs& a) {
     }
     if (a.out == SPH_OUT_BF16) return launch_degree_flags<float, float, __nv_bfloat16, DOWN, false>(a, tf);
     return launch_degree_flags<float, float, float, DOWN, false>(a, tf);
+#else
+    return int(cudaErrorInvalidValue);  // FP64 arithmetic only
+#endif
 }
 
 }  // namespace
@@ -556,8 +895,10 @@ int degree_fwd_down(const FwdArgs& a) { return degree_fwd_dir<true>(a); }
 int degree_fwd_up1(const FwdArgs& a) { return degree_fwd_dir<false>(a); }
 #elif SPH_DEGREE_LPP == 2
 int degree_fwd_up2(const FwdArgs& a) { return degree_fwd_dir<false>(a); }
-#else
+#elif SPH_DEGREE_LPP == 4
 int degree_fwd_up4(const FwdArgs& a) { return degree_fwd_dir<false>(a); }
+#else
+int degree_fwd_up8(const FwdArgs& a) { return degree_fwd_dir<false>(a); }
 #endif
 
 }  // namespace sph

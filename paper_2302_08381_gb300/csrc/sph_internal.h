@@ -60,6 +60,13 @@ const void* device_tables(int dtype);
 // S = Qtilde_l^l on the diagonal.
 const void* device_tables_down(int dtype);
 
+// Tables of the DEGREE kernels with FP64 arithmetic (entry-major, kF64Tables
+// doubles per (l, m)): {A, B, S, f, e, 0, 0, 0}, A, B, S as above, f and e of the
+// m = 0 column without its 1/sqrt2.
+constexpr int kF64Tables = 8;
+const void* device_tables_f64();
+bool device_tables_f64_ready();  // already uploaded to the current device
+
 // Coefficient streams of the ROW kernels, FP32 (see sph_capi.cu): entry
 // (degree, slot, lane), lane fastest, kRowDegrees x kRowSlots x kRowLanes
 // float4 entries {A, B, S, e}, then as many floats f, then as many float4
@@ -199,6 +206,7 @@ size_t point_row_bytes(int L, int grad, int elem, int hess = 0);
 int degree_fwd_up1(const FwdArgs& a);
 int degree_fwd_up2(const FwdArgs& a);
 int degree_fwd_up4(const FwdArgs& a);
+int degree_fwd_up8(const FwdArgs& a);  // FP64 arithmetic only
 int degree_fwd_down(const FwdArgs& a);
 
 // ROW kernels (FP32 arithmetic, 16 <= l_max <= 63, values and gradients):
