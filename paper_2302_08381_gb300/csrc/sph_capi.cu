@@ -402,23 +402,18 @@ bool point4_default(int L, int grad, int elem, int hess, int hc, int normalized)
            (elem == 4 || L >= 9);  // bf16 at l_max 8: one lane 4.17, four 3.78 TB/s
 }
 
-sph_launch default_point_bwd(int L, int elem, int dbw) {
+// Whole 32-point tiles (the recursion runs on full warps). Small tiles in blocks
+// of two warps on a grid of 32 blocks per SM scheduled in waves (fused backward,
+// l_max 6: 11 % above a persistent one-wave grid; double backward, waves against
+// one wave, l_max 4 150 / 162 us, 8 324 / 350), except for the double backward
+// with even K (l_max 7 345 / 320) or three buffers of more than 12 KB (6 283 /
+// 257); larger tiles, and few of them, one warp per block and one wave.
+sph_launch default_point_bwd(int L, int elem, int dbw, int64_t n) {
     const size_t K = size_t(L + 1) * (L + 1);
-    const size_t V = (K % 2 == 0) ? K + 1 : K;
-    const int mult = tile_multiple(L, elem);
-    const size_t per_pt = V * elem * (dbw ? 3 : 2);
-    const size_t budget = 48 * 1024;
-    int P = 32;
-    while (P > mult && size_t(P) * per_pt > budget) P -= mult;
-    P = std::max(mult, P / mult * mult);
-    const size_t tile = size_t(P) * per_pt;
-    // Measured on GB300 (fused backward, l_max 6, 4.19M points): 2-warp CTAs
-    // on a grid of 32 CTAs per SM scheduled in waves beat the persistent
-    // one-wave grid by 11 % for small rows; the double backward is
-    // insensitive to the shape.
-    if (!dbw && tile <= 24 * 1024) return sph_launch{P, 2, 32, 0};
-    int W = int(std::max<size_t>(1, std::min<size_t>(4, budget / std::max<size_t>(tile, 1))));
-    return sph_launch{P, W, 0, 0};
+    const size_t row = (K % 2 == 0 ? K * elem + 16 : K * elem), tile = 32 * row;
+    const bool wave = dbw && (K % 2 == 0 || (3 * tile > 12 * 1024 && 3 * tile <= 21 * 1024));
+    if (2 * tile <= 24 * 1024 && n >= 128 * int64_t(sm_count())) return sph_launch{32, 2, wave ? 0 : 32, 0};
+    return sph_launch{32, 1, 0, 0};
 }
 
 // Validates / completes a POINT launch shape; returns false with a message.
@@ -923,7 +918,7 @@ static int backward_common(const void* xyz, const void* g, const void* v, int64_
         }
         const size_t K = size_t(l_max + 1) * (l_max + 1);
         const size_t V = (K % 2 == 0) ? K + 1 : K;  // padded smem rows for even K
-        if (!resolve_point(a.launch, default_point_bwd(l_max, e, dbw), l_max, e, V * e * (dbw ? 3 : 2)))
+        if (!resolve_point(a.launch, default_point_bwd(l_max, e, dbw, n), l_max, e, V * e * (dbw ? 3 : 2)))
             return SPH_EINVAL;
         PointBwdFn fn = dbw ? point_dbwd_fn(l_max) : point_bwd_fn(l_max);
         return cuda_status(fn(a), dbw ? "POINT double-backward launch" : "POINT backward launch");

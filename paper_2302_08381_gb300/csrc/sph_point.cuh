@@ -1018,7 +1018,8 @@ constexpr uint32_t kWaitPolls = 1u << 22;  // bounded mbarrier wait (>> any real
 //   dQ_l^m = (x dx + y dy) e Q_{l-1}^{m+1} + dz f Q_{l-1}^m,
 //   dA = m (dx B + dy C),  dB, dC from dc_{m-1}, ds_{m-1} likewise,
 // and every column's own derivative along that direction, dQ c_m + Q dc_m and
-// dQ s_m + Q ds_m, replaces its upstream gradient's slot in `orow`. That is
+// dQ s_m + Q ds_m, goes to `orow` (which may be `row` itself: a column's upstream
+// gradients are read before its outputs are written). That is
 // the double backward (grad_xyz is the derivative of the gradient along v,
 // grad_g the derivative of Y along v) without any Hessian entry: 37 operations
 // per pair of columns (17 without DUAL) where the six Hessian entries of both
@@ -1032,7 +1033,7 @@ struct ChanSums {
 
 template <int L, bool NORM, bool DUAL, typename T, typename Tabs>
 __device__ __forceinline__ void point_chan_sums(T x, T y, T z, T r2, T dx, T dy, T dz, const Tabs& tb,
-                                                const T* __restrict__ gr, T* __restrict__ orow, ChanSums<T>& a) {
+                                                const T* row, T* orow, ChanSums<T>& a) {
     T c[L + 1], s[L + 1];
     point_cs<L>(x, y, c, s);
     const T w = DUAL ? x * dx + y * dy : T(0);
@@ -1064,7 +1065,7 @@ __device__ __forceinline__ void point_chan_sums(T x, T y, T z, T r2, T dx, T dy,
             }
             const int k = l * l + l;
             if (m == 0) {
-                const T g = gr[k];
+                const T g = row[k];
                 a.P += E1 * g;
                 a.Z += Qz * g;
                 if (NORM) sl += (tb.inv_sqrt2 * q[0]) * g;
@@ -1076,7 +1077,7 @@ __device__ __forceinline__ void point_chan_sums(T x, T y, T z, T r2, T dx, T dy,
                     p[0] = dq * (T(2) * tb.inv_sqrt2);
                 }
             } else {
-                const T gp = gr[k + m], gn = gr[k - m];
+                const T gp = row[k + m], gn = row[k - m];
                 const T c1 = c[m - 1], s1 = s[m - 1];
                 const T A = gp * c[m] + gn * s[m];
                 const T B = gp * c1 + gn * s1;
@@ -1125,14 +1126,60 @@ __device__ __forceinline__ void point_chan_sums(T x, T y, T z, T r2, T dx, T dy,
     }
 }
 
-template <int L, typename T>
-__host__ __device__ constexpr size_t point_bwd_buf_bytes(int P) {
-    return align16(size_t(P) * RowStride<L>::V * sizeof(T));
+// The same with outputs that are known to lie apart from the gradients.
+template <int L, bool NORM, bool DUAL, typename T, typename Tabs>
+__device__ __forceinline__ void point_chan_sums_apart(T x, T y, T z, T r2, T dx, T dy, T dz, const Tabs& tb,
+                                                      const T* __restrict__ row, T* __restrict__ orow,
+                                                      ChanSums<T>& a) {
+    point_chan_sums<L, NORM, DUAL>(x, y, z, r2, dx, dy, dz, tb, row, orow, a);
 }
 
-// DBW = false: backward (dxyz). DBW = true: double backward (grad_g, grad_xyz).
-// Shared memory per warp: two upstream-gradient buffers, (DBW) one grad_g
-// buffer, and two mbarriers.
+// Row of the staged upstream-gradient tile. Odd K: the image of the global range
+// (one bulk copy; an odd stride is free of bank conflicts). Even K (a multiple
+// of 4): rows of K plus 16 bytes, every one 16-byte aligned, filled by 16-byte
+// asynchronous copies; 32 lanes reading one column then meet 8 banks. (Padding
+// such rows to K + 1 and filling them with plain loads, waited for before each
+// tile, ran at 1.65 TB/s at l_max 7 and 0.9 at 11 where l_max 6 and 8 ran at 5.9.)
+template <int L, typename T>
+struct BwdRow {
+    static constexpr int K = (L + 1) * (L + 1);
+    static constexpr bool EVEN = K % 2 == 0;
+    static constexpr int EL16 = 16 / int(sizeof(T));
+    static constexpr int CR = K / EL16;  // 16-byte units of a row (even K)
+    // l_max 1 in FP32: a row is one 16-byte unit, which its lane moves itself, in
+    // rows of 5 words (4M points: 48 us through the asynchronous copies)
+    static constexpr bool ONE = EVEN && CR == 1;
+    static constexpr int S = ONE ? K + 1 : (EVEN ? K + EL16 : K);
+};
+
+template <int L, typename T>
+__host__ __device__ constexpr size_t point_bwd_buf_bytes(int P) {
+    return align16(size_t(P) * BwdRow<L, T>::S * sizeof(T));
+}
+
+// Tile buffers per warp: two (the next tile's gradients load during the current
+// one) while that leaves room for ten warps on an SM; beyond, one, refilled
+// after each tile with the next one prefetched into L2: full 32-point tiles
+// and twice the warps count for more (the recursion bounds these l_max).
+template <int L, typename T>
+__host__ __device__ constexpr int point_bwd_bufs() {
+    return 2 * point_bwd_buf_bytes<L, T>(32) <= 21 * 1024 ? 2 : 1;
+}
+// Whether the double backward stages grad_g in a buffer of its own (odd K,
+// where three buffers fit the same room): no load waits for its copy out. At
+// l_max 6 in place took 269..283 us against 267 (4M points).
+template <int L, bool DBW, typename T>
+__host__ __device__ constexpr bool point_bwd_apart() {
+    return DBW && !BwdRow<L, T>::EVEN && 3 * point_bwd_buf_bytes<L, T>(32) <= 21 * 1024;
+}
+template <int L, bool DBW, typename T>
+__host__ __device__ constexpr size_t point_bwd_warp_bytes(int P) {
+    return (point_bwd_bufs<L, T>() + (point_bwd_apart<L, DBW, T>() ? 1 : 0)) * point_bwd_buf_bytes<L, T>(P) + 16;
+}
+
+// DBW = false: backward (dxyz). DBW = true: double backward (grad_g, grad_xyz);
+// grad_g takes the place of g in the staged rows, or a buffer of its own.
+// Shared memory per warp: the tile buffers and two mbarriers.
 template <int L, bool NORM, bool DBW, typename T>
 __global__ void __launch_bounds__(256) point_bwd_kernel(const T* __restrict__ xyz, const T* __restrict__ g,
                                                         const T* __restrict__ v, int64_t n,
@@ -1140,26 +1187,21 @@ __global__ void __launch_bounds__(256) point_bwd_kernel(const T* __restrict__ xy
                                                         T* __restrict__ dxyz, T* __restrict__ grad_g,
                                                         T* __restrict__ grad_xyz, int P, int bulk_in,
                                                         int bulk_out, uint32_t* __restrict__ status) {
-    constexpr int K = (L + 1) * (L + 1);
-    using RS = RowStride<L>;
-    if constexpr (RS::PAD) bulk_in = bulk_out = 0;  // padded rows: plain loads / stores
-    (void)bulk_out;
+    using BR = BwdRow<L, T>;
+    constexpr int K = BR::K;
+    constexpr int NB = point_bwd_bufs<L, T>();
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int W = blockDim.x >> 5;
     const size_t buf = point_bwd_buf_bytes<L, T>(P);
-    const size_t per_warp = (DBW ? 3 : 2) * buf + 16;
-    unsigned char* base = smem + size_t(warp) * per_warp;
-    T* const sg0 = reinterpret_cast<T*>(base);
-    T* const sg1 = reinterpret_cast<T*>(base + buf);
-    T* so = reinterpret_cast<T*>(base + 2 * buf);
-    uint64_t* bar = reinterpret_cast<uint64_t*>(base + (DBW ? 3 : 2) * buf);
+    unsigned char* base = smem + size_t(warp) * point_bwd_warp_bytes<L, DBW, T>(P);
+    constexpr bool APART = point_bwd_apart<L, DBW, T>();
+    T* const so = reinterpret_cast<T*>(base + NB * buf);  // APART: grad_g
+    uint64_t* bar = reinterpret_cast<uint64_t*>(base + (NB + (APART ? 1 : 0)) * buf);
 
-    if (lane == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-    }
+    if (lane == 0)
+        for (int b = 0; b < NB; ++b) mbar_init(&bar[b], 1);
     fence_proxy_async_smem();
     __syncwarp();
 
@@ -1168,52 +1210,77 @@ __global__ void __launch_bounds__(256) point_bwd_kernel(const T* __restrict__ xy
     int64_t tile = int64_t(blockIdx.x) * W + warp;
     uint32_t phase = 0;    // bit b: parity of buffer b's next completion
     uint32_t pending = 0;  // bit b: a bulk load into buffer b is in flight
-    int64_t eb0 = 0, eb1 = 0;
     bool failed = false;
 
-    if (tile < ntiles) {
-        const int64_t p0 = tile * P;
+    // Starts loading a tile into buffer b (free: its readers are past a
+    // __syncwarp, bulk stores out of it have been waited for by lane 0).
+    auto load = [&](int64_t t, int b) {
+        const int64_t p0 = t * P;
         const int64_t cnt = min(int64_t(P), n - p0);
-        eb0 = issue_tile_load(sg0, g + p0 * K, cnt * K, bulk_in, &bar[0], lane);
-        if (eb0 > 0) pending |= 1u;
-    }
+        T* dst = reinterpret_cast<T*>(base + b * buf);
+        if constexpr (BR::EVEN && !BR::ONE) {
+            if (bulk_in) {
+                const T* src = g + p0 * K;
+                const uint32_t d0 = smem_u32(dst);
+                for (int i = lane; i < int(cnt) * BR::CR; i += 32)
+                    cp_async16(d0 + uint32_t((i / BR::CR) * BR::S * int(sizeof(T)) + (i % BR::CR) * 16), src + i * BR::EL16);
+            }
+        } else if constexpr (!BR::EVEN) {
+            if (issue_tile_load(dst, g + p0 * K, cnt * K, bulk_in, &bar[b], lane) > 0) pending |= 1u << b;
+        }
+    };
+
+    if (tile < ntiles) load(tile, 0);
+    cp_async_commit();
     int cur = 0;
     for (; tile < ntiles; tile += stride) {
         const int64_t p0 = tile * P;
         const int cnt = int(min(int64_t(P), n - p0));
-        // Prefetch the next tile into the other buffer; its previous contents
-        // were consumed in the last iteration, which ended with a proxy fence
-        // and __syncwarp.
         const int64_t nt = tile + stride;
-        const int nxt = cur ^ 1;
-        if (nt < ntiles) {
-            const int64_t q0 = nt * P;
-            const int64_t qc = min(int64_t(P), n - q0);
-            const int64_t e = issue_tile_load(nxt ? sg1 : sg0, g + q0 * K, qc * K, bulk_in, &bar[nxt], lane);
-            if (nxt) eb1 = e; else eb0 = e;
-            if (e > 0) pending |= (1u << nxt);
+        const int nxt = NB == 2 ? cur ^ 1 : 0;
+        if constexpr (NB == 2) {
+            if (DBW && !APART && lane == 0) bulk_wait_read_all();  // grad_g of the last tile has left the other buffer
+            if (nt < ntiles) load(nt, nxt);
+            cp_async_commit();
+        } else if (bulk_in && lane == 0 && nt < ntiles) {
+            const int64_t bytes = min(int64_t(P), n - nt * P) * K * int64_t(sizeof(T)) / 16 * 16;
+            if (bytes > 0) bulk_prefetch_l2(g + nt * P * K, uint32_t(bytes));
         }
-        // Wait for this tile's bulk part, then load the remainder directly.
-        if (pending & (1u << cur)) {
-            bool ok = true;
-            if (lane == 0) ok = mbar_wait_bounded(&bar[cur], (phase >> cur) & 1u, kWaitPolls);
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (ok) {
-                phase ^= (1u << cur);
-                pending &= ~(1u << cur);
-            } else {
-                if (lane == 0) atomicOr(status, kStatusLoadTimeout);
-                failed = true;
-            }
-        }
-        if (failed) break;
-        const int64_t eb_cur = cur ? eb1 : eb0;
-        T* const gt = cur ? sg1 : sg0;
-        if constexpr (RS::PAD) {
-            warp_rows_in<K>(gt, g + p0 * K, cnt, RS::V, lane);
+        T* const gt = reinterpret_cast<T*>(base + cur * buf);
+        if constexpr (BR::EVEN) {
+            if (bulk_in && BR::ONE) {
+                if (lane < cnt) {
+                    const float4 r = *reinterpret_cast<const float4*>(g + (p0 + lane) * K);
+                    T* const row = gt + lane * BR::S;
+                    row[0] = r.x;
+                    row[1] = r.y;
+                    row[2] = r.z;
+                    row[3] = r.w;
+                }
+            } else if (bulk_in)
+                cp_async_wait<NB - 1>();
+            else
+                warp_rows_in<K>(gt, g + p0 * K, cnt, BR::S, lane);
         } else {
-            for (int64_t i = eb_cur + lane; i < int64_t(cnt) * K; i += 32) gt[i] = g[p0 * K + i];
+            // Wait for this tile's bulk part, then load the remainder directly.
+            if (pending & (1u << cur)) {
+                bool ok = true;
+                if (lane == 0) ok = mbar_wait_bounded(&bar[cur], (phase >> cur) & 1u, kWaitPolls);
+                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                if (ok) {
+                    phase ^= (1u << cur);
+                    pending &= ~(1u << cur);
+                } else {
+                    if (lane == 0) atomicOr(status, kStatusLoadTimeout);
+                    failed = true;
+                }
+            }
+            if (failed) break;
+            const int64_t ev = int64_t(cnt) * K;
+            const int64_t eb = bulk_in ? ev * int64_t(sizeof(T)) / 16 * 16 / int64_t(sizeof(T)) : 0;
+            for (int64_t i = eb + lane; i < ev; i += 32) gt[i] = g[p0 * K + i];
         }
+        if (APART && lane == 0) bulk_wait_read_all();  // grad_g of the last tile has left its buffer
         __syncwarp();
         if (lane < cnt) {
             const int64_t p = p0 + lane;
@@ -1224,10 +1291,10 @@ __global__ void __launch_bounds__(256) point_bwd_kernel(const T* __restrict__ xy
             } else {
                 r2 = x * x + y * y + z * z;
             }
-            const T* gr = gt + size_t(lane) * RS::V;
+            T* const row = gt + size_t(lane) * BR::S;
             ChanSums<T> a;
             if constexpr (!DBW) {
-                point_chan_sums<L, NORM, false>(x, y, z, r2, T(0), T(0), T(0), tb, gr, static_cast<T*>(nullptr), a);
+                point_chan_sums<L, NORM, false>(x, y, z, r2, T(0), T(0), T(0), tb, row, row, a);
                 T ax = x * a.P + a.Bq, ay = y * a.P + a.Cq, az = a.Z;
                 if (NORM) {
                     ax = ir * (ax - x * a.S);
@@ -1247,7 +1314,10 @@ __global__ void __launch_bounds__(256) point_bwd_kernel(const T* __restrict__ xy
                     dy = ir * (dy - y * uv);
                     dz = ir * (dz - z * uv);
                 }
-                point_chan_sums<L, NORM, true>(x, y, z, r2, dx, dy, dz, tb, gr, so + size_t(lane) * RS::V, a);
+                if constexpr (APART)
+                    point_chan_sums_apart<L, NORM, true>(x, y, z, r2, dx, dy, dz, tb, row, so + size_t(lane) * BR::S, a);
+                else
+                    point_chan_sums<L, NORM, true>(x, y, z, r2, dx, dy, dz, tb, row, row, a);
                 if (grad_xyz) {
                     T hx = dx * a.P + x * a.dP + a.dB;
                     T hy = dy * a.P + y * a.dP + a.dC;
@@ -1268,33 +1338,52 @@ __global__ void __launch_bounds__(256) point_bwd_kernel(const T* __restrict__ xy
             }
         }
         if constexpr (DBW) {
-            if (grad_g && RS::PAD) {
-                __syncwarp();
-                warp_rows_out<K>(grad_g + p0 * K, so, cnt, RS::V, lane);
-            } else if (grad_g) {
+            if (grad_g) {
+                T* const out = grad_g + p0 * K;
+                const T* const src = APART ? so : gt;
                 fence_proxy_async_smem();
                 __syncwarp();
-                const int64_t ev = int64_t(cnt) * K;
-                int64_t eo = 0;
-                if (bulk_out) {
-                    eo = (ev * int64_t(sizeof(T))) / 16 * 16 / int64_t(sizeof(T));
-                    if (lane == 0 && eo > 0) {
-                        bulk_store(grad_g + p0 * K, so, uint32_t(eo * sizeof(T)));
-                        bulk_commit();
+                if constexpr (BR::EVEN) {
+                    if (bulk_out && BR::ONE) {
+                        const T* const row = gt + lane * BR::S;
+                        if (lane < cnt)
+                            *reinterpret_cast<float4*>(out + lane * K) =
+                                make_float4(float(row[0]), float(row[1]), float(row[2]), float(row[3]));
+                    } else if (bulk_out) {
+                        for (int i = lane; i < cnt * BR::CR; i += 32)
+                            reinterpret_cast<float4*>(out)[i] = *reinterpret_cast<const float4*>(
+                                gt + (i / BR::CR) * BR::S + (i % BR::CR) * BR::EL16);
+                    } else {
+                        warp_rows_out<K>(out, gt, cnt, BR::S, lane);
                     }
+                } else {
+                    const int64_t ev = int64_t(cnt) * K;
+                    int64_t eo = 0;
+                    if (bulk_out) {
+                        eo = (ev * int64_t(sizeof(T))) / 16 * 16 / int64_t(sizeof(T));
+                        if (lane == 0 && eo > 0) {
+                            bulk_store(out, src, uint32_t(eo * sizeof(T)));
+                            bulk_commit();
+                        }
+                    }
+                    for (int64_t i = eo + lane; i < ev; i += 32) out[i] = src[i];
                 }
-                for (int64_t i = eo + lane; i < ev; i += 32) grad_g[p0 * K + i] = so[i];
-                if (bulk_out && lane == 0) bulk_wait_read_all();
             }
         }
         fence_proxy_async_smem();
         __syncwarp();
+        if constexpr (NB == 1) {
+            if (DBW && lane == 0) bulk_wait_read_all();
+            if (nt < ntiles) load(nt, 0);
+            cp_async_commit();
+        }
         cur = nxt;
     }
+    cp_async_wait<0>();
     if (pending && lane == 0) {
         // Loads issued but never observed (after a timeout) may still be in
         // flight: wait for them, bounded, before the shared memory goes away.
-        for (int b = 0; b < 2; ++b)
+        for (int b = 0; b < NB; ++b)
             if (pending & (1u << b)) (void)mbar_wait_bounded(&bar[b], (phase >> b) & 1u, kWaitPolls);
     }
     if (DBW && lane == 0) bulk_wait_all();
@@ -1456,8 +1545,11 @@ int launch_point10_fwd(const FwdArgs& a) {
 template <int L, bool NORM, bool DBW, typename T>
 int launch_point_bwd(const BwdArgs& a) {
     static const PointTabs<L, T, false> tb = make_point_tabs<L, T, false>();
-    const int P = a.launch.points_per_tile, W = a.launch.warps_per_block;
-    const size_t smem = size_t(W) * ((DBW ? 3 : 2) * point_bwd_buf_bytes<L, T>(P) + 16);
+    const int P = a.launch.points_per_tile;
+    int W = a.launch.warps_per_block;
+    const size_t per_warp = point_bwd_warp_bytes<L, DBW, T>(P);
+    while (W > 1 && size_t(W) * per_warp > size_t(max_smem_optin())) --W;  // even K: rows wider than the shape's check
+    const size_t smem = size_t(W) * per_warp;
     auto kern = point_bwd_kernel<L, NORM, DBW, T>;
     cudaError_t err = ensure_smem(kern, smem);
     if (err != cudaSuccess) return int(err);
