@@ -78,7 +78,9 @@ typedef enum { SPH_OUT_SAME = 0, SPH_OUT_BF16 = 1 } sph_out;
 typedef enum { SPH_Q_NATIVE = 0, SPH_Q_F64 = 1 } sph_qprec;
 
 /* Kernel family. AUTO picks, by measurement on GB300: DEGREE for FP64
- * arithmetic without Hessians (the mixed mode; SPH_F64 from l_max 14, with
+ * arithmetic without Hessians (the mixed mode, except with FP32 storage to
+ * l_max 4, from l_max 3 on 8,192 points or more: POINT_HC with FP64
+ * arithmetic; SPH_F64 from l_max 14, with
  * gradients from l_max 9, and by the number of points from l_max 11, with
  * gradients 5: launch_info, which takes none, reports the choice for few
  * points); else

@@ -550,6 +550,14 @@ bool point_hybrid_wins(int l_max, int dtype, bool grad) {
 
 namespace {
 
+// FP64 arithmetic on FP32 storage at small l_max: POINT_HC's one lane per point,
+// whole rows by bulk copies, against DEGREE's stage of a few degrees (400k
+// points, gradients, us: l_max 1 89 on DEGREE, 17 for POINT_HC in FP64; 2 140 /
+// 27; 3 189 / 70; 4 275 / 136; 5 357 / 240, but the conversions of the outputs run
+// on the FP64 pipe in POINT, 144 per point there). Few points: DEGREE's split of
+// a point over lanes from l_max 3.
+bool mixed_prefers_point(int64_t n, int l_max) { return l_max <= kMixedHcMaxL && (l_max <= 2 || n >= 8192); }
+
 // FP64 requests below auto_family's DEGREE limits that run faster there all
 // the same, by the number of points. Measured on GB300 (us, POINT / DEGREE):
 // gradients, normalized (scaled), 400k points l_max 6 601 / 531 (365 / 440), 7
@@ -694,6 +702,12 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
             cudaGetLastError();
     }
     int hc = 0;
+    const bool mixed_point = kernel == SPH_KERNEL_AUTO && !launch && mixed && !ddsph && out == SPH_OUT_SAME &&
+                             mixed_prefers_point(n, l_max);
+    if (mixed_point) {
+        fam = SPH_KERNEL_POINT;
+        hc = 1;
+    }
     if (fam == SPH_KERNEL_POINT_HC) {
         if (l_max > kHcMaxL || ddsph || mixed || out != SPH_OUT_SAME) {
             set_error("POINT_HC takes l_max <= %d, values and gradients, native Q precision and same-type storage",
@@ -703,7 +717,7 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
         hc = 1;
         fam = SPH_KERNEL_POINT;
     }
-    if (fam == SPH_KERNEL_POINT && (l_max > SPH_MAX_L_POINT || hess_bf16 || mixed)) {
+    if (fam == SPH_KERNEL_POINT && !mixed_point && (l_max > SPH_MAX_L_POINT || hess_bf16 || mixed)) {
         set_error("POINT kernels take l_max <= %d, native Q precision, and no bf16 Hessians", SPH_MAX_L_POINT);
         return SPH_EUNSUPPORTED;
     }
@@ -738,7 +752,7 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
     a.hc = hc;
     if (fam == SPH_KERNEL_POINT) {
         bool from_default = !launch;
-        if (!launch) {
+        if (!launch && !mixed_point) {
             int d = -1;
             cudaGetDevice(&d);
             std::lock_guard<std::mutex> lk(g_mu);

@@ -148,6 +148,9 @@ inline int point4_default_warps(int L) { return point4_out_mode(L, 4) == 1 ? 2 :
 
 // Largest l_max with the hybrid POINT forward (hard-coded l <= 3) compiled.
 constexpr int kHcMaxL = 8;
+// ... and compiled for FP64 arithmetic on FP32 storage (AUTO's choice there, see
+// mixed_prefers_point).
+constexpr int kMixedHcMaxL = 4;
 
 // Whether AUTO runs the hybrid instead of the all-recursion POINT forward
 // (values, or values and gradients; no Hessians).

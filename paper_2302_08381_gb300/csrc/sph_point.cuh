@@ -22,6 +22,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 
 #include "sph_core.cuh"
@@ -253,8 +254,13 @@ __device__ __forceinline__ void warp_rows_in(T* __restrict__ sdst, const T* __re
     }
 }
 
+// Type of the coordinates: the arithmetic's, but FP32 for FP64 arithmetic on
+// FP32 storage.
+template <typename T, typename TO>
+using PointIn = std::conditional_t<sizeof(T) == 8 && sizeof(TO) != 8, float, T>;
+
 template <int L, bool GRAD, bool HESS, bool NORM, typename T, typename TO, bool HC = false>
-__global__ void __launch_bounds__(256) point_fwd_kernel(const T* __restrict__ xyz, int64_t n,
+__global__ void __launch_bounds__(256) point_fwd_kernel(const PointIn<T, TO>* __restrict__ xyz, int64_t n,
                                                         const __grid_constant__ PointTabs<L, T, HESS> tb,
                                                         TO* __restrict__ sph, TO* __restrict__ dsph,
                                                         TO* __restrict__ ddsph, int P, int bulk) {
@@ -1479,7 +1485,7 @@ int launch_point_fwd(const FwdArgs& a) {
                       (!GRAD || reinterpret_cast<uintptr_t>(a.dsph) % 16 == 0) &&
                       (!HESS || reinterpret_cast<uintptr_t>(a.ddsph) % 16 == 0);
     kern<<<grid, 32 * W, smem, static_cast<cudaStream_t>(a.stream)>>>(
-        static_cast<const T*>(a.xyz), a.n, tb, static_cast<TO*>(a.sph), static_cast<TO*>(a.dsph),
+        static_cast<const PointIn<T, TO>*>(a.xyz), a.n, tb, static_cast<TO*>(a.sph), static_cast<TO*>(a.dsph),
         static_cast<TO*>(a.ddsph), P, bulk ? 1 : 0);
     return int(cudaGetLastError());
 }

@@ -53,6 +53,12 @@ int SPH_CAT(point_fwd_L, SPH_INST_L)(const FwdArgs& a) {
             if (a.dtype == SPH_F64) {
                 SPH_FWD_HC(double, double)
             }
+            if (a.qprec == SPH_Q_F64) {  // FP64 arithmetic on FP32 storage
+                if constexpr (L <= kMixedHcMaxL) {
+                    SPH_FWD_HC(double, float)
+                }
+                return int(cudaErrorInvalidValue);
+            }
             SPH_FWD_HC(float, float)
 #undef SPH_FWD_HC
         }
