@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "sph_core.cuh"
 #include "sph_internal.h"
@@ -82,6 +83,23 @@ __device__ __forceinline__ CSf row_power(const CSf& w1, const CSf& w2, const CSf
     const CSf r4 = r.times(w4);
     if (e & 4) r = r4;
     return r;
+}
+
+// Calls f with the compile-time number of channel slots, kend + 1 <= N, that a
+// degree uses: every slot but the last is then full (no lane masked, no
+// branch), and the slots of a degree interleave. The backward is 4..10 % faster
+// for it (l_max 20, 200k points: 175 -> 162 us; 30, 100k: 179 -> 167); the
+// forward, with its eight stores per slot, is not (l_max 40..63 up to 10 % slower).
+template <int N, int K = 0, typename F>
+__device__ __forceinline__ void row_slots(int kend, F&& f) {
+    if constexpr (K + 1 < N) {
+        if (kend == K)
+            f(std::integral_constant<int, K + 1>{});
+        else
+            row_slots<N, K + 1>(kend, f);
+    } else {
+        f(std::integral_constant<int, N>{});
+    }
 }
 
 // Coefficients in shared memory, once per block: entry (degree, slot, lane) of
@@ -503,38 +521,34 @@ __global__ void __launch_bounds__(32 * kRowBwdWarps, 1) row_bwd_kernel(
                 const float* const gp0 = gb + (ctr - s0 + kBPad + j);  // + 8k: g of column ctr + m
                 const float* const gn0 = gb + (ctr - s0 + kBPad - j);
                 float sd = 0.f;
-                auto next_q = [&](int k) {
-                    const float src = (j == 0) ? (k + 1 < NCH ? q1[k + 1 < NCH ? k + 1 : k] : 0.f) : q1[k];
-                    return __shfl_sync(0xffffffffu, src, nb_lane);
-                };
-                float4 tn = dA[0];
-                float fn = dF[0], qnn = next_q(0);
+                row_slots<NCH>(kend, [&](auto ks) {
+                    constexpr int KS = decltype(ks)::value;
+                    float qn[KS];
 #pragma unroll
-                for (int k = 0; k < NCH; ++k) {
-                    if (k > kend) break;
-                    const float4 t0 = tn;
-                    const float f0 = fn, qn = qnn;
-                    if (k + 1 < NCH) {
-                        tn = dA[(k + 1) * kRowLanes];
-                        fn = dF[(k + 1) * kRowLanes];
-                        qnn = next_q(k + 1);
+                    for (int k = 0; k < KS; ++k) {
+                        const float src = (j == 0) ? (k + 1 < NCH ? q1[k + 1 < NCH ? k + 1 : k] : 0.f) : q1[k];
+                        qn[k] = __shfl_sync(0xffffffffu, src, nb_lane);
                     }
-                    // zero for m > d: the table holds zeros there
-                    const float q = fmaf(t0.x * z, q1[k], fmaf(-(t0.y * r2), q2[k], t0.z));
-                    if (j + kG * k <= d) {
-                        const float gp = gp0[kG * k], gn = gn0[-kG * k];
-                        const float A = fmaf(gp, cm[k], gn * sm[k]);        // g+ c_m + g- s_m
-                        const float B = fmaf(gp, cm1[k], gn * sm1[k]);      // m (g+ c_{m-1} + g- s_{m-1})
-                        const float Cc = fmaf(gn, cm1[k], -(gp * sm1[k]));  // m (g- c_{m-1} - g+ s_{m-1})
-                        P = fmaf(t0.w * qn, A, P);
-                        Bq = fmaf(q, B, Bq);
-                        Cq = fmaf(q, Cc, Cq);
-                        Z = fmaf(f0 * q1[k], A, Z);
-                        if (NORM) sd = fmaf(q, A, sd);
+#pragma unroll
+                    for (int k = 0; k < KS; ++k) {
+                        const float4 t0 = dA[k * kRowLanes];
+                        // zero for m > d: the table holds zeros there
+                        const float q = fmaf(t0.x * z, q1[k], fmaf(-(t0.y * r2), q2[k], t0.z));
+                        if (k + 1 < KS || j + kG * k <= d) {
+                            const float gp = gp0[kG * k], gn = gn0[-kG * k];
+                            const float A = fmaf(gp, cm[k], gn * sm[k]);        // g+ c_m + g- s_m
+                            const float B = fmaf(gp, cm1[k], gn * sm1[k]);      // m (g+ c_{m-1} + g- s_{m-1})
+                            const float Cc = fmaf(gn, cm1[k], -(gp * sm1[k]));  // m (g- c_{m-1} - g+ s_{m-1})
+                            P = fmaf(t0.w * qn[k], A, P);
+                            Bq = fmaf(q, B, Bq);
+                            Cq = fmaf(q, Cc, Cq);
+                            Z = fmaf(dF[k * kRowLanes] * q1[k], A, Z);
+                            if (NORM) sd = fmaf(q, A, sd);
+                        }
+                        q2[k] = q1[k];
+                        q1[k] = q;
                     }
-                    q2[k] = q1[k];
-                    q1[k] = q;
-                }
+                });
                 if (NORM) S = fmaf(float(d), sd, S);
             }
             fence_proxy_async_smem();  // this buffer is rewritten by the async proxy two windows on
