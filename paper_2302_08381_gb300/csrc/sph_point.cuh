@@ -361,36 +361,42 @@ __global__ void __launch_bounds__(256) point_fwd_kernel(const PointIn<T, TO>* __
 // 8 to 16 points. Every lane runs the Q recursion (Eq. iter-q) and Eq.
 // iter-sc in full (cheap next to the assembly) and assembles only its plane
 // with role weights, the same instruction stream in every lane:
-//   plane = A c_m + m Qtilde_l^m C'_m,   A = a0 Qtilde + ax e Qtilde_{l-1}^{m+1} + a3 f Qtilde_{l-1}^m
-// (a0, ax, a3) = (1, 0, 0), (0, x, 0), (0, y, 0), (0, 0, 1) by role, and
-// C'_m = c_{m-1} (d/dx), -s_{m-1} (d/dy), 0 (value, d/dz); the sin-type column
-// takes s_m and S'_m = s_{m-1}, c_{m-1}, 0. These are the terms of Eq.
-// iter-deri that assemble_m combines for all four planes at once.
+//   plane = A c_m + Qtilde_l^m C'_m,   A = aq Qtilde + ax e Qtilde_{l-1}^{m+1} + a3 f Qtilde_{l-1}^m
+// (aq, ax, a3) = (1, 0, 0), (0, x, 0), (0, y, 0), (0, 0, 1) by role, and
+// C'_m = m c_{m-1} (d/dx), -m s_{m-1} (d/dy), 0 (value, d/dz); the sin-type column
+// takes s_m and S'_m = m s_{m-1}, m c_{m-1}, 0. These are the terms of Eq.
+// iter-deri that assemble_m combines for all four planes at once. The
+// normalized form, (plane - l u_r Y) / r, has the same terms: 1/r goes into ax,
+// a3 and C', S', and -l u_r / r into aq. 13 operations per pair of columns;
+// with m and the normalization applied to the assembled columns it was 14, and
+// 20 normalized, and bf16 rows and normalized l_max >= 12 are bound by them
+// (issue 75 % busy at l_max 10, bf16).
 template <int L, bool NORM, typename T, typename TO, typename Tabs>
 __device__ __forceinline__ void point4_core(T x, T y, T z, T r2, const Tabs& tb, int r, T ir,
                                             TO* __restrict__ rowp) {
+    const T irr = (NORM && r != 0) ? ir : T(1);
     const T a0 = r == 0 ? T(1) : T(0);
-    const T ax = r == 1 ? x : (r == 2 ? y : T(0));
-    const T a3 = r == 3 ? T(1) : T(0);
-    const T a00 = a0 * tb.inv_sqrt2;  // m = 0 value: Qtilde_l^0 / sqrt2
+    const T ax = irr * (r == 1 ? x : (r == 2 ? y : T(0)));
+    const T a3 = r == 3 ? irr : T(0);
+    const T nu = NORM ? -irr * (r == 1 ? x : (r == 2 ? y : (r == 3 ? z : T(0)))) : T(0);  // l times: into aq
     T c[L + 1], s[L + 1];
     point_cs<L>(x, y, c, s);
+    // The factor m is in (C'_m, S'_m), except in the scaled form to l_max 12, where
+    // multiplying Qtilde by it measured 2..3 % faster (bf16; l_max 14, 16: 9 % slower)
+    constexpr bool FOLD = NORM || L > 12;
+    auto fm = [](int m) { return FOLD ? T(m) : T(1); };
     T c1[L + 1], s1[L + 1];  // (C'_m, S'_m) of this lane's role
     {
-        const T k1 = r == 1 ? T(1) : T(0), k2 = r == 2 ? T(-1) : T(0);
-        const T k3 = r == 2 ? T(1) : T(0), k4 = r == 1 ? T(1) : T(0);
+        const T k1 = r == 1 ? irr : T(0), k2 = r == 2 ? -irr : T(0);
+        const T k3 = r == 2 ? irr : T(0), k4 = r == 1 ? irr : T(0);
         c1[0] = T(0);
         s1[0] = T(0);
 #pragma unroll
         for (int m = 1; m <= L; ++m) {
-            c1[m] = k1 * c[m - 1] + k2 * s[m - 1];
-            s1[m] = k3 * c[m - 1] + k4 * s[m - 1];
+            c1[m] = fm(m) * (k1 * c[m - 1] + k2 * s[m - 1]);
+            s1[m] = fm(m) * (k3 * c[m - 1] + k4 * s[m - 1]);
         }
     }
-    // Normalized form (x, y, z = u): plane' = irr (plane - l u_r value), with
-    // u_r = 0 and irr = 1 for the value plane.
-    const T nu = NORM ? -(r == 1 ? x : (r == 2 ? y : (r == 3 ? z : T(0)))) : T(0);
-    const T irr = (NORM && r != 0) ? ir : T(1);
     T q1[L + 1], q2[L + 1];
 #pragma unroll
     for (int m = 0; m <= L; ++m) {
@@ -407,27 +413,19 @@ __device__ __forceinline__ void point4_core(T x, T y, T z, T r2, const Tabs& tb,
             const int i = tri(l, m);
             q[m] = (tb.a[i] * z) * q1[m] - (tb.b[i] * r2) * q2[m];
         }
-        const T nl = nu * T(l);
+        const T aq = NORM ? fma(nu, T(l), a0) : a0;
 #pragma unroll
         for (int m = 0; m <= l; ++m) {
             const int i = tri(l, m);
             const T E1 = (m + 1 <= l - 1) ? tb.e[i] * q1[m + 1] : T(0);
             const T Qz = (m <= l - 1) ? tb.fz[i] * q1[m] : T(0);
             if (m == 0) {
-                T out = a00 * q[0] + ax * E1 + a3 * Qz;
-                if (NORM) out = irr * fma(nl, q[0] * tb.inv_sqrt2, out);
-                rowp[l * l + l] = OutConv<TO>::cv(out);
+                rowp[l * l + l] = OutConv<TO>::cv((aq * tb.inv_sqrt2) * q[0] + ax * E1 + a3 * Qz);
             } else {
-                const T A = a0 * q[m] + ax * E1 + a3 * Qz;
-                const T mQ = T(m) * q[m];
-                T oc = A * c[m] + mQ * c1[m];
-                T os = A * s[m] + mQ * s1[m];
-                if (NORM) {
-                    oc = irr * fma(nl, q[m] * c[m], oc);
-                    os = irr * fma(nl, q[m] * s[m], os);
-                }
-                rowp[l * l + l + m] = OutConv<TO>::cv(oc);
-                rowp[l * l + l - m] = OutConv<TO>::cv(os);
+                const T A = aq * q[m] + ax * E1 + a3 * Qz;
+                const T mq = FOLD ? q[m] : T(m) * q[m];
+                rowp[l * l + l + m] = OutConv<TO>::cv(A * c[m] + mq * c1[m]);
+                rowp[l * l + l - m] = OutConv<TO>::cv(A * s[m] + mq * s1[m]);
             }
         }
 #pragma unroll
