@@ -678,21 +678,22 @@ __device__ __forceinline__ void point16_core(float x, float y, float z, float r2
                 }
             } else {
                 const float Am = aQl * q[m] + A;
-                const float mB = float(m) * (bQ * q[m] + bE * E1 + bz * Qz);
-                const float mq = float(m) * q[m];
+                const float B = bQ * q[m] + bE * E1 + bz * Qz;
                 const float c1 = c[m - 1], s1 = s[m - 1];
                 const float c2 = m >= 2 ? c[m >= 2 ? m - 2 : 0] : 0.f, s2 = m >= 2 ? s[m >= 2 ? m - 2 : 0] : 0.f;
-                float oc = Am * c[m] + mB * (k1c * c1 + k1s * s1);
-                float os = Am * s[m] + mB * (k2c * c1 + k2s * s1);
+                // role columns of m alone (the same for every l), with its factors m, m (m - 1)
+                const float t1c = float(m) * (k1c * c1 + k1s * s1), t1s = float(m) * (k2c * c1 + k2s * s1);
+                const float t2c = float(m * (m - 1)) * (k3c * c2 + k3s * s2);
+                const float t2s = float(m * (m - 1)) * (k4c * c2 + k4s * s2);
+                float oc = Am * c[m] + B * t1c;
+                float os = Am * s[m] + B * t1s;
                 if (NORM) {
-                    const float Uc = float(l) * (k5 * c1 - k6 * s1) + float(m - 1) * (k3c * c2 + k3s * s2);
-                    const float Us = float(l) * (k5 * s1 + k6 * c1) + float(m - 1) * (k4c * c2 + k4s * s2);
-                    oc += mq * Uc;
-                    os += mq * Us;
+                    const float t3c = float(m) * (k5 * c1 - k6 * s1), t3s = float(m) * (k5 * s1 + k6 * c1);
+                    oc += q[m] * (float(l) * t3c + t2c);
+                    os += q[m] * (float(l) * t3s + t2s);
                 } else if (m >= 2) {
-                    const float MQ = float(m - 1) * mq;
-                    oc += MQ * (k3c * c2 + k3s * s2);
-                    os += MQ * (k4c * c2 + k4s * s2);
+                    oc += q[m] * t2c;
+                    os += q[m] * t2s;
                 }
                 if (store) {
                     rowp[l * l + l + m] = oc;
