@@ -14,9 +14,10 @@
 // Range: a factor of exponent within 2^+-300 (Mul64) and operands within
 // 2^+-700, so every product is a normal number; zeros, subnormals, infinities,
 // NaN and the rest of the range are reported, and the caller repeats the work
-// on the FP64 pipe. It does so for a whole step of its loop in one branch: a
-// branch around one or two FP64 instructions is compiled to predication, and
-// a predicated-off FP64 instruction still takes its turn on the pipe.
+// on the FP64 pipe. It does so for a whole step of its loop in one branch:
+// with a branch around every pair of products the kernel was no faster than on
+// the FP64 pipe alone (DEGREE, l_max 30, 200k points: 5.6 ms, and 4.4 with one
+// branch per step).
 #pragma once
 
 #include <cuda_runtime.h>
