@@ -1378,7 +1378,10 @@ __global__ void __launch_bounds__(256) point_bwd_kernel(const T* __restrict__ xy
         fence_proxy_async_smem();
         __syncwarp();
         if constexpr (NB == 1) {
-            if (DBW && lane == 0) bulk_wait_read_all();
+            if constexpr (DBW) {
+                if (lane == 0) bulk_wait_read_all();
+                __syncwarp();  // no lane refills the buffer (plain loads, g not 16-byte aligned) before grad_g has left it
+            }
             if (nt < ntiles) load(nt, 0);
             cp_async_commit();
         }
