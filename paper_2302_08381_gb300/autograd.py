@@ -5,6 +5,7 @@ backward (for force training) is the double-backward kernel."""
 from __future__ import annotations
 
 import torch
+from torch.autograd import forward_ad
 from torch.autograd.function import once_differentiable
 
 from . import api
@@ -46,7 +47,9 @@ class SphericalHarmonicsFn(torch.autograd.Function):
         (xyz,) = ctx.saved_tensors
         if not ctx.needs_input_grad[0]:
             return None, None, None
-        if not torch.is_grad_enabled() and type(g) is torch.Tensor and not torch._C._functorch.is_functorch_wrapped_tensor(g):
+        plain = type(g) is torch.Tensor and not torch._C._functorch.is_functorch_wrapped_tensor(g)
+        # (within a dual level g may carry a tangent, which only a node can refuse)
+        if plain and not torch.is_grad_enabled() and forward_ad._current_level < 0:
             # no graph of the backward is asked for: without the second node the
             # step of 2,561 points at l_max 4 takes 30 us less host time
             return api.backward(xyz, g, ctx.l_max, ctx.normalized), None, None
