@@ -486,22 +486,25 @@ struct F64Step {
     double xc, xs, yc, ys, zc, zs;  // gradient planes of both columns
 };
 
-// FAST: the products that are not part of an fma on the integer pipe; returns
-// false where one of them has an operand out of its range (the caller then
-// repeats the step without FAST). A product with a factor that is zero by its
+// Where the products that are not part of an fma are done.
+enum class Mul { kFp64, kInt, kIntZero };
+
+// kInt, kIntZero: those products on the integer pipe; returns false where one of
+// them has an operand out of its range (the caller then repeats the step with
+// kFp64; kIntZero takes zeros too). A product with a factor that is zero by its
 // place (s_0, Q_{l-1}^{m+1} beyond the degree) is no such case: it is set to
 // zero. t: {A, B, S, f}, e; q: {Qtilde_{l-1}^m, Qtilde_{l-2}^m}; qr:
 // Qtilde_{l-1}^{m+1}; c, ci, c1: {c_m, s_m}, the same / r, m {c_{m-1}, s_{m-1}} / r.
-template <bool FAST, bool GRAD, bool NORM>
+template <Mul MUL, bool GRAD, bool NORM>
 __device__ __forceinline__ bool f64_step(int l, int m, const double4_32a& t, double e, const F64Point& P, double lx,
                                          double ly, double lz, const double2& q, double qr, const double2& c,
                                          const double2& ci, const double2& c1, F64Step& o) {
     bool in = true;
     // a * b, or 0 where it is not `used`
     auto mul = [&](double a, const Mul64& b, bool used) {
-        if (!FAST) return used ? a * b.v : 0.0;
+        if constexpr (MUL == Mul::kFp64) return used ? a * b.v : 0.0;
         bool ok = b.ok;
-        const double p = b.fast(a, ok);
+        const double p = b.template fast<MUL == Mul::kIntZero>(a, ok);
         in = in && (ok || !used);
         return used ? p : 0.0;
     };
@@ -567,11 +570,12 @@ __device__ __forceinline__ bool f64_put(TO* __restrict__ st, int sp, int sm, con
 // channels, the same number in every lane of the warp; lanes with m > l only
 // take part in the shuffle. `st64`: this lane's state, pair i of slot k at
 // [32 (i NS + k)]; `qc` carries {q1, q2} of the lane's current channel.
-template <int LPP, bool GRAD, bool NORM, typename TO>
+// `fp64` (the same in every lane): straight to the FP64 pipe.
+template <Mul MUL, int LPP, bool GRAD, bool NORM, typename TO>
 __device__ __forceinline__ void f64_chunk(int l, int m_lo, int m_hi, int h, int lane, int sp0, int sm0,
                                           const double* __restrict__ tab, const F64Point& P, double lx, double ly,
-                                          double lz, double2* __restrict__ st64, int NS, TO* __restrict__ st,
-                                          double2& qc) {
+                                          double lz, bool fp64, double2* __restrict__ st64, int NS,
+                                          TO* __restrict__ st, double2& qc) {
     constexpr int PL = (32 / LPP) * (2 * kMC64<TO, GRAD> + 1);
     constexpr unsigned kAll = 0xffffffffu;
     const int up = (lane & ~(LPP - 1)) | ((h + 1) & (LPP - 1));  // the lane of channel m + 1
@@ -596,8 +600,10 @@ __device__ __forceinline__ void f64_chunk(int l, int m_lo, int m_hi, int h, int 
             if (LPP > 1) qr = __shfl_sync(kAll, h == 0 ? qn.x : qc.x, up);
         }
         F64Step o;
-        const bool in = f64_step<true, GRAD, NORM>(l, m, t0, e, P, lx, ly, lz, qc, qr, c, ci, c1, o);
-        if (__any_sync(kAll, on && !in)) f64_step<false, GRAD, NORM>(l, m, t0, e, P, lx, ly, lz, qc, qr, c, ci, c1, o);
+        bool in = false;
+        if (!fp64) in = f64_step<MUL, GRAD, NORM>(l, m, t0, e, P, lx, ly, lz, qc, qr, c, ci, c1, o);
+        if (__any_sync(kAll, on && !in))
+            f64_step<Mul::kFp64, GRAD, NORM>(l, m, t0, e, P, lx, ly, lz, qc, qr, c, ci, c1, o);
         if (on) st64[32 * k] = make_double2(o.q, qc.x);
         if (sizeof(TO) == 8) {
             f64_put<false, PL, GRAD>(st, sp0 + m, sm0 - m, o, on);
@@ -608,13 +614,59 @@ __device__ __forceinline__ void f64_chunk(int l, int m_lo, int m_hi, int h, int 
     }
 }
 
+// Everything after the prologue: degrees 0..L of a tile.
+template <Mul MUL, int LPP, bool GRAD, bool NORM, typename TO>
+__device__ __forceinline__ void f64_tile(int L, bool fp64, int h, int lane, const double* __restrict__ tab, const F64Point& P,
+                                         double2* __restrict__ st64, int NS, TO* __restrict__ stw,
+                                         TO* __restrict__ stl, TO* __restrict__ sph_t, TO* __restrict__ dsph_t,
+                                         int64_t K, int np) {
+    constexpr int PPW = 32 / LPP, MC = kMC64<TO, GRAD>, ST = 2 * MC + 1;
+    const double x = P.x, y = P.y, z = P.z.v;
+    int l = 0;
+    while (l <= L) {
+        if (2 * l + 1 <= 2 * MC) {
+            // Whole small degrees la..lb, contiguous columns la^2 .. (lb+1)^2-1.
+            const int la = l;
+            int lb = l;
+            while (lb < L && (lb + 2) * (lb + 2) - la * la <= 2 * MC) ++lb;
+            const int colA0 = la * la;
+            for (int d = la; d <= lb; ++d) {
+                const int c0 = d * d + d - colA0;
+                const double dl = double(d);
+                double2 qc = st64[0];
+                f64_chunk<MUL, LPP, GRAD, NORM>(d, 0, d, h, lane, c0, c0, tab, P, dl * x, dl * y, dl * z, fp64, st64,
+                                                NS, stl, qc);
+            }
+            const int nc = (lb + 1) * (lb + 1) - colA0;
+            flush_stage<PPW, GRAD, ST>(stw, sph_t, dsph_t, K, np, nc, nc, colA0, colA0, lane);
+            l = lb + 1;
+        } else {
+            const int ctr = l * l + l;
+            const double dl = double(l);
+            const double lx = dl * x, ly = dl * y, lz = dl * z;
+            double2 qc = st64[0];
+            for (int m_lo = 0; m_lo <= l; m_lo += MC) {
+                const int m_hi = min(l, m_lo + MC - 1);
+                const int colA0 = ctr - m_hi;
+                const int nA = m_lo == 0 ? 2 * m_hi + 1 : m_hi - m_lo + 1;
+                const int nc = m_lo == 0 ? nA : 2 * nA;
+                const int offB = m_lo == 0 ? colA0 : ctr + m_lo - nA;
+                f64_chunk<MUL, LPP, GRAD, NORM>(l, m_lo, m_hi, h, lane, ctr - offB, ctr - colA0, tab, P, lx, ly, lz,
+                                                fp64, st64, NS, stl, qc);
+                flush_stage<PPW, GRAD, ST>(stw, sph_t, dsph_t, K, np, nc, nA, colA0, offB, lane);
+            }
+            ++l;
+        }
+    }
+}
+
 template <typename TI, typename TO, bool GRAD, bool NORM, int LPP>
 __global__ void __launch_bounds__(256, 2) degree_f64_kernel(const TI* __restrict__ xyz, int64_t n, int L,
                                                                            const double* __restrict__ tab,
                                                                            double inv_sqrt2, TO* __restrict__ sph,
                                                                            TO* __restrict__ dsph) {
     constexpr int PPW = 32 / LPP;  // points per warp tile
-    constexpr int MC = kMC64<TO, GRAD>, ST = 2 * MC + 1;
+    constexpr int ST = 2 * kMC64<TO, GRAD> + 1;
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -632,12 +684,10 @@ __global__ void __launch_bounds__(256, 2) degree_f64_kernel(const TI* __restrict
     for (int64_t tile = int64_t(blockIdx.x) * W + warp; tile < ntiles; tile += int64_t(gridDim.x) * W) {
         const int64_t p0 = tile * PPW;
         const int np = int(min(int64_t(PPW), n - p0));
-        double x = 0.0, y = 0.0, z = 0.0, ir = 1.0;
-        if (pt < np) {
-            x = double(xyz[3 * (p0 + pt)]);
-            y = double(xyz[3 * (p0 + pt) + 1]);
-            z = double(xyz[3 * (p0 + pt) + 2]);
-        }
+        // (the lanes past the last point run on it: its operands are as good as any)
+        const TI* const xp = xyz + 3 * (p0 + min(pt, np - 1));
+        double x = double(xp[0]), y = double(xp[1]), z = double(xp[2]), ir = 1.0;
+        const bool zeros = __any_sync(0xffffffffu, x == 0.0 || y == 0.0 || z == 0.0);
         if (NORM) {  // u = xyz / r, r2 = |u|^2 of the rounded u (0 at r = 0), as in unit_point
             const double rr = fma(x, x, fma(y, y, z * z));
             ir = rr > 0.0 ? 1.0 / sqrt(rr) : 0.0;
@@ -673,42 +723,18 @@ __global__ void __launch_bounds__(256, 2) degree_f64_kernel(const TI* __restrict
             }
         }
 
-        int l = 0;
-        while (l <= L) {
-            if (2 * l + 1 <= 2 * MC) {
-                // Whole small degrees la..lb, contiguous columns la^2 .. (lb+1)^2-1.
-                const int la = l;
-                int lb = l;
-                while (lb < L && (lb + 2) * (lb + 2) - la * la <= 2 * MC) ++lb;
-                const int colA0 = la * la;
-                for (int d = la; d <= lb; ++d) {
-                    const int c0 = d * d + d - colA0;
-                    const double dl = double(d);
-                    double2 qc = st64[0];
-                    f64_chunk<LPP, GRAD, NORM>(d, 0, d, h, lane, c0, c0, tab, P, dl * x, dl * y, dl * z, st64, NS, stl,
-                                               qc);
-                }
-                const int nc = (lb + 1) * (lb + 1) - colA0;
-                flush_stage<PPW, GRAD, ST>(stw, sph_t, dsph_t, K, np, nc, nc, colA0, colA0, lane);
-                l = lb + 1;
-            } else {
-                const int ctr = l * l + l;
-                const double dl = double(l);
-                const double lx = dl * x, ly = dl * y, lz = dl * z;
-                double2 qc = st64[0];
-                for (int m_lo = 0; m_lo <= l; m_lo += MC) {
-                    const int m_hi = min(l, m_lo + MC - 1);
-                    const int colA0 = ctr - m_hi;
-                    const int nA = m_lo == 0 ? 2 * m_hi + 1 : m_hi - m_lo + 1;
-                    const int nc = m_lo == 0 ? nA : 2 * nA;
-                    const int offB = m_lo == 0 ? colA0 : ctr + m_lo - nA;
-                    f64_chunk<LPP, GRAD, NORM>(l, m_lo, m_hi, h, lane, ctr - offB, ctr - colA0, tab, P, lx, ly, lz,
-                                               st64, NS, stl, qc);
-                    flush_stage<PPW, GRAD, ST>(stw, sph_t, dsph_t, K, np, nc, nA, colA0, offB, lane);
-                }
-                ++l;
-            }
-        }
+        // A point with a zero coordinate has a zero Qtilde, c_m or s_m at every
+        // second step, and trying those steps on the integer pipe first cost more than
+        // it gains (200k points with z = 0, us, with the trial / now: values, l_max 12
+        // 354 / 239, 20 885 / 600; gradients, l_max 8 659 / 537, 20 3063 / 2433). Values
+        // take a copy of the loop whose products accept zeros. With gradients a copy
+        // is too much code (on the FP64 pipe, tiles of both kinds at l_max 12: 1126
+        // against 1005 us), so those tiles take the FP64 pipe in the same loop.
+        if (GRAD || !zeros)
+            f64_tile<Mul::kInt, LPP, GRAD, NORM>(L, GRAD && zeros, h, lane, tab, P, st64, NS, stw, stl, sph_t, dsph_t, K,
+                                                 np);
+        else if constexpr (!GRAD)
+            f64_tile<Mul::kIntZero, LPP, GRAD, NORM>(L, false, h, lane, tab, P, st64, NS, stw, stl, sph_t, dsph_t, K, np);
     }
 }
 #endif

@@ -12,12 +12,13 @@
 // FP64 pipe every product that is not part of an fma is moved here.
 //
 // Range: a factor of exponent within 2^+-300 (Mul64) and operands within
-// 2^+-700, so every product is a normal number; zeros, subnormals, infinities,
-// NaN and the rest of the range are reported, and the caller repeats the work
-// on the FP64 pipe. It does so for a whole step of its loop in one branch:
-// with a branch around every pair of products the kernel was no faster than on
-// the FP64 pipe alone (DEGREE, l_max 30, 200k points: 5.6 ms, and 4.4 with one
-// branch per step).
+// 2^+-700, so every product is a normal number; subnormals, infinities, NaN and
+// the rest of the range are reported, and the caller repeats the work on the
+// FP64 pipe. It does so for a whole step of its loop in one branch: with a
+// branch around every pair of products the kernel was no faster than on the FP64
+// pipe alone (DEGREE, l_max 30, 200k points: 5.6 ms, and 4.4 with one branch per
+// step). A zero operand is reported too, unless ZERO: a test and two selects per
+// product, taken for tiles with a point that has a zero coordinate.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -31,7 +32,8 @@ struct Mul64 {
     uint32_t hi;      // its high word (sign, exponent)
     uint32_t m1, m0;  // significand, shifted left to fill 64 bits
     uint32_t ex;      // exponent field minus that of 2^1
-    bool ok;
+    bool ok;    // in range
+    bool zero;  // +-0
 
     __device__ __forceinline__ explicit Mul64(double b) : v(b) {
         hi = uint32_t(__double2hiint(b));
@@ -40,15 +42,21 @@ struct Mul64 {
         m0 = lo << 11;
         const uint32_t e = hi & 0x7ff00000u;
         ok = e - ((1023u - 300u) << 20) <= (600u << 20);
+        zero = ((hi & 0x7fffffffu) | lo) == 0u;
         ex = e - (1024u << 20);
     }
 
-    // a * v; `in` is cleared when a is out of the fast range (the result is
-    // then meaningless).
+    // a * v; `in` (the caller's `ok`) is cleared when a is out of the fast range:
+    // the result is then meaningless. ZERO: both ranges checked here, 0 in them.
+    template <bool ZERO>
     __device__ __forceinline__ double fast(double a, bool& in) const {
         const uint32_t ah = uint32_t(__double2hiint(a)), al = uint32_t(__double2loint(a));
         const uint32_t ea = ah & 0x7ff00000u;
-        in = in && ea - ((1023u - 700u) << 20) <= (1400u << 20);
+        const bool az = ZERO && ((ah & 0x7fffffffu) | al) == 0u;
+        if constexpr (ZERO)
+            in = (ok || zero) && (az || ea - ((1023u - 700u) << 20) <= (1400u << 20));
+        else
+            in = in && ea - ((1023u - 700u) << 20) <= (1400u << 20);
         const uint32_t am = (ah & 0x000fffffu) | 0x00100000u;
         // the product of the 53-bit and the 64-bit significand, 117 bits: hi:l1:l0
         const uint64_t t0 = uint64_t(al) * m0;
@@ -64,7 +72,8 @@ struct Mul64 {
         const uint32_t up = ((H0 >> 1) & 1u) | (((l1 << s) | l0) != 0u ? 1u : 0u);
         const uint64_t R = ((uint64_t(H1) << 32) | H0) + up;
         const uint32_t rh = uint32_t(R >> 33) + ea + ex + (n << 20);  // a carry out of the significand moves the exponent
-        return __hiloint2double(int(rh | ((ah ^ hi) & 0x80000000u)), int(uint32_t(R >> 1)));
+        const bool nz = !(ZERO && (az || zero));
+        return __hiloint2double(int((nz ? rh : 0u) | ((ah ^ hi) & 0x80000000u)), int(nz ? uint32_t(R >> 1) : 0u));
     }
 };
 
