@@ -529,12 +529,15 @@ int degree_default_lpp(int l_max, int dtype, int qprec) {
 // l_max 50 12.6/7.4/5.4; values, 200k l_max 12 .23/.25/-, 20 .60/.55/-, 30
 // 1.7/1.1/-; 100k l_max 40 1.9/1.15/-, 50 2.7/2.0/1.6. Few points: enough lanes
 // for about six warps per SM (10k points, gradients, l_max 20 at 2 / 4 / 8 lanes:
-// 181/134/167 us; 1k points 248/97/72 us).
+// 181/134/167 us; 1k points 248/97/72 us). A point of l_max below 7 has few
+// channels to share out, and none for more than l_max + 1 lanes: FP32 values,
+// l_max 3, 4k points, 5.7/5.3/8.0 us, FP64 gradients, l_max 6, scaled, 10k points
+// 24.7/24.2/-, 4k -/15.0/18.6, 1k -/14.4/13.2.
 int degree_f64_lpp(int64_t n, int l_max, bool grad, bool mixed) {
     int lpp;
     if (grad) lpp = l_max > 26 ? 8 : (l_max >= (mixed ? 16 : 12) ? 4 : 2);
     else lpp = l_max > 44 ? 8 : (l_max >= 20 ? 4 : 2);
-    while (lpp < 8 && n * lpp < int64_t(6) * 32 * sm_count()) lpp *= 2;
+    while (lpp < 8 && lpp <= l_max && n * lpp < int64_t(l_max < 7 ? 8 / lpp : 6) * 32 * sm_count()) lpp *= 2;
     return lpp;
 }
 
@@ -559,14 +562,18 @@ namespace {
 bool mixed_prefers_point(int64_t n, int l_max) { return l_max <= kMixedHcMaxL && (l_max <= 2 || n >= 8192); }
 
 // FP64 requests below auto_family's DEGREE limits that run faster there all
-// the same, by the number of points. Measured on GB300 (us, POINT / DEGREE):
-// gradients, normalized (scaled), 400k points l_max 6 601 / 531 (365 / 440), 7
-// 1172 / 623 (703 / 525); 300k l_max 8 1195 / 639 (697 / 496); 1k points l_max 4
-// 19 / 17, 5..8 33..52 / 21..27; values, 200k points l_max 12 248 / 224; 50k
-// l_max 10 52 / 62; 10k l_max 12 29 / 31.
-bool f64_prefers_degree(int64_t n, int l_max, bool grad) {
-    if (grad) return n >= 256 && (l_max >= 7 || (l_max >= 5 && n <= 8192));
-    return n >= 32768 && l_max >= 11;
+// the same, by the number of points. Measured on GB300, us, POINT / DEGREE.
+// Gradients, scaled: l_max 5 1k points 14.2/11.9, 4k 14.2/12.8, 8k 14.1/15.1; 6 4k
+// 17.6/15.0, 8k 18.6/17.7; 7 1k 24/14, 8k 24.0/20.3, 10k 24.2/26.3 (POINT's tiles
+// fill one wave there: 8 likewise, 30.4/33.7), 16k 46/31, 100k 166/151; 8 8k
+// 29.1/26.2, 16k 56/39, 100k 223/197. Normalized: 5 8k 23.0/18.2, 100k 116/119; 6 8k
+// 29.2/21.0; 7 10k 39/31, 100k 272/177. Values: 11 32k 46/40, 100k 100/90; 12 16k
+// 26.2/27.6, 32k 49/46; 13 16k 29.8/30.8, 100k 174/128; 10 100k 78/79.
+bool f64_prefers_degree(int64_t n, int l_max, bool grad, bool normalized) {
+    if (!grad) return n >= 32768 && l_max >= 11;
+    if (n < 256) return false;
+    if (l_max >= 7) return normalized || n <= 8192 || n > 12288;
+    return l_max >= 5 && n <= (normalized ? 8192 : 4096);
 }
 
 // AUTO kernel family of a forward request (measured on GB300). POINT
@@ -691,7 +698,7 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
     const bool hess_bf16 = ddsph && out == SPH_OUT_BF16;
     if (fam == SPH_KERNEL_AUTO)
         fam = auto_family(l_max, dtype, out, qprec, ddsph != nullptr, dsph != nullptr, normalized, n);
-    if (kernel == SPH_KERNEL_AUTO && !launch && dtype == SPH_F64 && !ddsph && f64_prefers_degree(n, l_max, grad)) {
+    if (kernel == SPH_KERNEL_AUTO && !launch && dtype == SPH_F64 && !ddsph && f64_prefers_degree(n, l_max, grad, normalized)) {
         // POINT needs no device tables: a call captured before any upload stays there
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (device_tables_f64_ready() ||

@@ -797,7 +797,12 @@ int launch_f64(const FwdArgs& a, const double* tb) {
         size_t(a.launch.warps_per_block) * degree_warp_bytes<kLPP, double, TO, GRAD, false>(a.l_max) > optin)
         return int(cudaErrorInvalidConfiguration);
     if (kLPP == 1 && per_warp > optin) return degree_fwd_up2(a);
-    int W = a.launch.warps_per_block > 0 ? a.launch.warps_per_block : default_warps(per_warp);
+    const int64_t ntiles = (a.n + PPW - 1) / PPW;
+    // Few tiles, up to eight per SM, in one-warp blocks: they spread evenly (gradients,
+    // scaled, l_max 8, 8k points 28.6 us in blocks of 4 warps, 26.2 so; 16k 51.4, 38.7;
+    // at 8.2 tiles per SM l_max 8 0.95, 20 1.04, 40 1.09 times the time).
+    const int few = ntiles <= int64_t(8) * sm_count() ? 1 : 4;
+    int W = a.launch.warps_per_block > 0 ? a.launch.warps_per_block : std::min(few, default_warps(per_warp));
     W = int(std::min<size_t>(W, optin / per_warp));
     const size_t smem = size_t(W) * per_warp;
     if (smem > 48 * 1024) {
@@ -816,7 +821,6 @@ int launch_f64(const FwdArgs& a, const double* tb) {
         }
         bps = std::max(occ, 1);
     }
-    const int64_t ntiles = (a.n + PPW - 1) / PPW;
     const int64_t want = (ntiles + W - 1) / W;
     const int grid = int(std::max<int64_t>(1, std::min<int64_t>(want, int64_t(bps) * sm_count())));
     kern<<<grid, 32 * W, smem, static_cast<cudaStream_t>(a.stream)>>>(
