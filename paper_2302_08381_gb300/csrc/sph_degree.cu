@@ -602,7 +602,7 @@ __device__ __forceinline__ void f64_chunk(int l, int m_lo, int m_hi, int h, int 
         F64Step o;
         bool in = false;
         if (!fp64) in = f64_step<MUL, GRAD, NORM>(l, m, t0, e, P, lx, ly, lz, qc, qr, c, ci, c1, o);
-        if (__any_sync(kAll, on && !in))
+        if (MUL != Mul::kFp64 && __any_sync(kAll, on && !in))
             f64_step<Mul::kFp64, GRAD, NORM>(l, m, t0, e, P, lx, ly, lz, qc, qr, c, ci, c1, o);
         if (on) st64[32 * k] = make_double2(o.q, qc.x);
         if (sizeof(TO) == 8) {
@@ -727,14 +727,17 @@ __global__ void __launch_bounds__(256, 2) degree_f64_kernel(const TI* __restrict
         // second step, and trying those steps on the integer pipe first cost more than
         // it gains (200k points with z = 0, us, with the trial / now: values, l_max 12
         // 354 / 239, 20 885 / 600; gradients, l_max 8 659 / 537, 20 3063 / 2433). Values
-        // take a copy of the loop whose products accept zeros. With gradients a copy
-        // is too much code (on the FP64 pipe, tiles of both kinds at l_max 12: 1126
-        // against 1005 us), so those tiles take the FP64 pipe in the same loop.
-        if (GRAD || !zeros)
-            f64_tile<Mul::kInt, LPP, GRAD, NORM>(L, GRAD && zeros, h, lane, tab, P, st64, NS, stw, stl, sph_t, dsph_t, K,
+        // take a copy of the loop whose products accept zeros. With gradients that is
+        // too much code; those tiles run on the FP64 pipe alone, scaled in a copy of
+        // the loop (a flag in the one loop: random points 1..5 % slower), normalized
+        // by the flag (a copy: tiles of both kinds at l_max 12 1126 us, 1005 so).
+        constexpr bool FLAG = GRAD && NORM;
+        if (FLAG || !zeros)
+            f64_tile<Mul::kInt, LPP, GRAD, NORM>(L, FLAG && zeros, h, lane, tab, P, st64, NS, stw, stl, sph_t, dsph_t, K,
                                                  np);
-        else if constexpr (!GRAD)
-            f64_tile<Mul::kIntZero, LPP, GRAD, NORM>(L, false, h, lane, tab, P, st64, NS, stw, stl, sph_t, dsph_t, K, np);
+        else if constexpr (!FLAG)
+            f64_tile<GRAD ? Mul::kFp64 : Mul::kIntZero, LPP, GRAD, NORM>(L, false, h, lane, tab, P, st64, NS, stw, stl,
+                                                                        sph_t, dsph_t, K, np);
     }
 }
 #endif
