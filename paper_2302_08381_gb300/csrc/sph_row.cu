@@ -146,10 +146,16 @@ __device__ __forceinline__ void row_table_ready() {
 // with c'_m = m c_{m-1} (and 1/r) folded into the kept c_{m-1}: 22 floating-point
 // operations per slot instead of 30.
 constexpr int kRowMaxWarps = 2;  // of an explicit launch shape
-SPH_HD constexpr int row_block_warps(int NCH) { return NCH <= 5 ? 12 : (NCH == 6 ? 10 : (NCH == 7 ? 9 : 8)); }
+// bfloat16 rows take half the shared memory, so the registers are the limit (50k
+// points, l_max 20: 79.7 us with 12 warps, 73.9 with 16; l_max 40, 244 with 10, 199 with 14).
+template <typename TO>
+SPH_HD constexpr int row_block_warps(int NCH) {
+    if (sizeof(TO) == 2 && NCH <= 6) return NCH <= 5 ? 16 : 14;
+    return NCH <= 5 ? 12 : (NCH == 6 ? 10 : (NCH == 7 ? 9 : 8));
+}
 
 template <typename TO, bool GRAD, bool NORM, int NCH, bool MINRUN>
-__global__ void __launch_bounds__(32 * row_block_warps(NCH), 1) row_fwd_kernel(const float* __restrict__ xyz, int64_t n,
+__global__ void __launch_bounds__(32 * row_block_warps<TO>(NCH), 1) row_fwd_kernel(const float* __restrict__ xyz, int64_t n,
                                                       int L, const float4* __restrict__ rowA,
                                                       const float* __restrict__ rowF, float inv_sqrt2,
                                                       TO* __restrict__ sph, TO* __restrict__ dsph) {
@@ -587,6 +593,15 @@ __global__ void __launch_bounds__(32 * kRowBwdWarps, 1) row_bwd_kernel(
     __syncwarp();
 }
 
+// Warps of the one block per SM: every one that fits (`fit`), but no more than
+// the rounds of tiles need. With the largest block the last round can fall on few
+// SMs (10k points, l_max 31, 2,500 tiles: 12 warps on each SM, then 57 SMs with 12
+// more, 49.1 us; two rounds of 9 39.8; before the blocks of many warps 45.6).
+int row_even_warps(int64_t tiles, int64_t fit) {
+    const int64_t spread = (tiles + sm_count() - 1) / sm_count(), rounds = (spread + fit - 1) / fit;
+    return int(std::max<int64_t>(1, (spread + rounds - 1) / std::max<int64_t>(rounds, 1)));
+}
+
 template <typename TO, bool GRAD, bool NORM, int NCH, bool MINRUN>
 int launch_row(const FwdArgs& a) {
     const float* rt = static_cast<const float*>(device_row_tables());
@@ -597,10 +612,7 @@ int launch_row(const FwdArgs& a) {
     int W = a.launch.warps_per_block;
     if (W > kRowMaxWarps) return int(cudaErrorInvalidConfiguration);
     if (W <= 0) {
-        // one block per SM with every warp that fits; few tiles are spread over the SMs
-        const int64_t fit = int64_t((size_t(max_smem_optin()) - table) / per_warp);
-        const int64_t spread = (tiles + sm_count() - 1) / sm_count();
-        W = int(std::max<int64_t>(1, std::min<int64_t>({int64_t(row_block_warps(NCH)), fit, spread})));
+        W = row_even_warps(tiles, std::min<int64_t>(row_block_warps<TO>(NCH), (size_t(max_smem_optin()) - table) / per_warp));
     }
     const size_t smem = table + size_t(W) * per_warp;
     if (smem > size_t(max_smem_optin())) return int(cudaErrorInvalidConfiguration);
@@ -637,9 +649,7 @@ int launch_row_bwd(const BwdArgs& a) {
     const int64_t tiles = (a.n + kPW - 1) / kPW;
     int W = a.launch.warps_per_block;
     if (W <= 0) {
-        const int64_t fit = int64_t((size_t(max_smem_optin()) - table) / per_warp);
-        const int64_t spread = (tiles + sm_count() - 1) / sm_count();
-        W = int(std::max<int64_t>(1, std::min<int64_t>({int64_t(kRowBwdWarps), fit, spread})));
+        W = row_even_warps(tiles, std::min<int64_t>(kRowBwdWarps, (size_t(max_smem_optin()) - table) / per_warp));
     }
     const size_t smem = table + size_t(W) * per_warp;
     if (smem > size_t(max_smem_optin())) return int(cudaErrorInvalidConfiguration);
