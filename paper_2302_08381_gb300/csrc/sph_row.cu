@@ -602,39 +602,52 @@ int row_even_warps(int64_t tiles, int64_t fit) {
     return int(std::max<int64_t>(1, (spread + rounds - 1) / std::max<int64_t>(rounds, 1)));
 }
 
+// The default: one such block per SM. An explicit shape of warps_per_block x
+// blocks_per_sm runs as many warps on an SM, in one block that shares the table as
+// long as they fit: a table for each of the caller's one- or two-warp blocks
+// leaves room for few of them (50k points, normalized, 1 x 0, us: l_max 50 1048, in
+// one block 405; 63 1679, 608).
+struct RowShape {
+    int W, grid;
+    size_t smem;
+};
+
+int row_shape(const void* kern, int64_t n, int cap, size_t per_warp, size_t table, const sph_launch& s, RowShape* r) {
+    const int64_t tiles = (n + kPW - 1) / kPW;
+    const int64_t fit = std::min<int64_t>(cap, (size_t(max_smem_optin()) - table) / per_warp);
+    const int64_t asked = int64_t(s.warps_per_block) * s.blocks_per_sm;  // 0: as many as fit
+    r->W = row_even_warps(tiles, asked > 0 ? std::min(asked, fit) : fit);
+    r->smem = table + size_t(r->W) * per_warp;
+    if (r->smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(r->smem));
+        if (e != cudaSuccess) return int(e);
+    }
+    int64_t bps = asked > 0 ? std::max<int64_t>(1, asked / r->W) : s.blocks_per_sm;
+    if (bps <= 0) {
+        int occ = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * r->W, r->smem) != cudaSuccess) {
+            cudaGetLastError();
+            occ = 1;
+        }
+        bps = std::max(occ, 1);
+    }
+    r->grid = int(std::max<int64_t>(1, std::min<int64_t>((tiles + r->W - 1) / r->W, bps * sm_count())));
+    return int(cudaSuccess);
+}
+
 template <typename TO, bool GRAD, bool NORM, int NCH, bool MINRUN>
 int launch_row(const FwdArgs& a) {
     const float* rt = static_cast<const float*>(device_row_tables());
     if (!rt) return int(cudaErrorMemoryAllocation);
     auto kern = row_fwd_kernel<TO, GRAD, NORM, NCH, MINRUN>;
     const size_t per_warp = row_warp_bytes<TO, GRAD, NCH, MINRUN>(), table = row_table_bytes<NCH>(a.l_max);
-    const int64_t tiles = (a.n + kPW - 1) / kPW;
-    int W = a.launch.warps_per_block;
-    if (W > kRowMaxWarps) return int(cudaErrorInvalidConfiguration);
-    if (W <= 0) {
-        W = row_even_warps(tiles, std::min<int64_t>(row_block_warps<TO>(NCH), (size_t(max_smem_optin()) - table) / per_warp));
-    }
-    const size_t smem = table + size_t(W) * per_warp;
-    if (smem > size_t(max_smem_optin())) return int(cudaErrorInvalidConfiguration);
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kern),
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return int(e);
-    }
-    int bps = a.launch.blocks_per_sm;
-    if (bps <= 0) {
-        int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, reinterpret_cast<const void*>(kern), 32 * W, smem) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            occ = 1;
-        }
-        bps = std::max(occ, 1);
-    }
-    const int64_t want = (tiles + W - 1) / W;
-    const int grid = int(std::max<int64_t>(1, std::min<int64_t>(want, int64_t(bps) * sm_count())));
+    if (a.launch.warps_per_block > kRowMaxWarps) return int(cudaErrorInvalidConfiguration);
+    RowShape r;
+    const int e = row_shape(reinterpret_cast<const void*>(kern), a.n, row_block_warps<TO>(NCH), per_warp, table,
+                            a.launch, &r);
+    if (e != int(cudaSuccess)) return e;
     constexpr int kEntries = kRowLanes * kRowDegrees * kRowSlots;
-    kern<<<grid, 32 * W, smem, static_cast<cudaStream_t>(a.stream)>>>(
+    kern<<<r.grid, 32 * r.W, r.smem, static_cast<cudaStream_t>(a.stream)>>>(
         static_cast<const float*>(a.xyz), a.n, a.l_max, reinterpret_cast<const float4*>(rt), rt + 4 * kEntries,
         float(host_tables().inv_sqrt2), static_cast<TO*>(a.sph), static_cast<TO*>(a.dsph));
     return int(cudaGetLastError());
@@ -646,32 +659,12 @@ int launch_row_bwd(const BwdArgs& a) {
     if (!rt) return int(cudaErrorMemoryAllocation);
     auto kern = row_bwd_kernel<NORM, NCH>;
     const size_t per_warp = row_bwd_warp_bytes(), table = row_table_bytes<NCH>(a.l_max);
-    const int64_t tiles = (a.n + kPW - 1) / kPW;
-    int W = a.launch.warps_per_block;
-    if (W <= 0) {
-        W = row_even_warps(tiles, std::min<int64_t>(kRowBwdWarps, (size_t(max_smem_optin()) - table) / per_warp));
-    }
-    const size_t smem = table + size_t(W) * per_warp;
-    if (smem > size_t(max_smem_optin())) return int(cudaErrorInvalidConfiguration);
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kern),
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return int(e);
-    }
-    int bps = a.launch.blocks_per_sm;
-    if (bps <= 0) {
-        int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, reinterpret_cast<const void*>(kern), 32 * W, smem) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            occ = 1;
-        }
-        bps = std::max(occ, 1);
-    }
-    const int64_t want = (tiles + W - 1) / W;
-    const int grid = int(std::max<int64_t>(1, std::min<int64_t>(want, int64_t(bps) * sm_count())));
+    RowShape r;
+    const int e =
+        row_shape(reinterpret_cast<const void*>(kern), a.n, kRowBwdWarps, per_warp, table, a.launch, &r);
+    if (e != int(cudaSuccess)) return e;
     constexpr int kEntries = kRowLanes * kRowDegrees * kRowSlots;
-    kern<<<grid, 32 * W, smem, static_cast<cudaStream_t>(a.stream)>>>(
+    kern<<<r.grid, 32 * r.W, r.smem, static_cast<cudaStream_t>(a.stream)>>>(
         static_cast<const float*>(a.xyz), static_cast<const float*>(a.g), a.n, a.l_max,
         reinterpret_cast<const float4*>(rt), rt + 4 * kEntries, float(host_tables().inv_sqrt2), static_cast<float*>(a.dxyz), a.status);
     return int(cudaGetLastError());
