@@ -660,8 +660,10 @@ __device__ __forceinline__ void f64_tile(int L, bool fp64, int h, int lane, cons
     }
 }
 
+// Blocks of up to 8 warps, at most 128 registers; values 96 (the bound for two
+// blocks of 10 warps), which leaves 20 warps on an SM.
 template <typename TI, typename TO, bool GRAD, bool NORM, int LPP>
-__global__ void __launch_bounds__(256, 2) degree_f64_kernel(const TI* __restrict__ xyz, int64_t n, int L,
+__global__ void __launch_bounds__(GRAD ? 256 : 320, 2) degree_f64_kernel(const TI* __restrict__ xyz, int64_t n, int L,
                                                                            const double* __restrict__ tab,
                                                                            double inv_sqrt2, TO* __restrict__ sph,
                                                                            TO* __restrict__ dsph) {
@@ -699,28 +701,56 @@ __global__ void __launch_bounds__(256, 2) degree_f64_kernel(const TI* __restrict
         TO* const sph_t = sph + p0 * K;
         TO* const dsph_t = GRAD ? dsph + p0 * 3 * K : nullptr;
 
-        {  // (x + i y)^m of this lane's channels (Eq. iter-sc), steps of (x + i y)^LPP; the recursion state zeroed
-            const CS<double> xy{x, y};
-            CS<double> a{1.0, 0.0}, b{1.0, 0.0}, w{1.0, 0.0};  // ^m, ^(m-1) (h = 0: ^(m+LPP-1))
-#pragma unroll
-            for (int t = 0; t < LPP; ++t) {
-                if (t < h) a = a.times(xy);
-                if (t < (h > 0 ? h - 1 : LPP - 1)) b = b.times(xy);
-                w = w.times(xy);
+        {  // (x + i y)^m of this lane's channels (Eq. iter-sc), the recursion state zeroed
+            // ^e for e < 8 by its bits, then steps of ^8: the same products, and so the same
+            // bits, for every LPP, which AUTO chooses by the number of points. Slot by slot in
+            // shared memory: eight powers in registers took values from 96 to 106 (l_max 30,
+            // 100k points: 537 -> 605 us).
+            constexpr int RB = 8 / LPP;  // slots per step of ^8
+            const CS<double> xy{x, y}, w2 = xy.times(xy), w4 = w2.times(w2), w8 = w4.times(w4);
+            double2* const cs = st64 + 32 * NS;
+            auto put = [&](int k, const CS<double>& v) { cs[32 * k] = make_double2(v.c, v.s); };
+            auto get = [&](int k) { return CS<double>{cs[32 * k].x, cs[32 * k].y}; };
+            CS<double> a{1.0, 0.0};  // ^h
+            if (h & 1) a = xy;
+            if (LPP > 2) {
+                const CS<double> t = a.times(w2);
+                if (h & 2) a = t;
             }
+            if (LPP > 4) {
+                const CS<double> t = a.times(w4);
+                if (h & 4) a = t;
+            }
+            put(0, a);
+#pragma unroll
+            for (int n1 = 1; n1 < RB; n1 *= 2)
+#pragma unroll
+                for (int r = 0; r < n1; ++r)
+                    if (n1 + r < NS) put(n1 + r, LPP * n1 == 1 ? xy : get(r).times(LPP * n1 == 2 ? w2 : w4));
+#pragma unroll 1
+            for (int k = RB; k < NS; ++k) {
+                a = (RB > 1 ? get(k - RB) : a).times(w8);
+                put(k, a);
+            }
+            // c_{m-1}: the lane below holds it, for lane 0 the last one, a slot earlier
+            const double2* const below = cs + (h > 0 ? -1 : LPP - 1 - 32);
+            if (LPP > 1) __syncwarp();
+#pragma unroll 1
             for (int k = 0; k < NS; ++k) {
                 const bool m0 = k == 0 && h == 0;
-                const double2 c = make_double2(m0 ? inv_sqrt2 : a.c, a.s);
                 st64[32 * k] = make_double2(0.0, 0.0);
-                st64[32 * (NS + k)] = c;
                 if (GRAD) {
-                    const double f = m0 ? 0.0 : double(h + LPP * k) * ir;
-                    st64[32 * (2 * NS + k)] = make_double2(f * b.c, f * b.s);
-                    if (NORM) st64[32 * (3 * NS + k)] = make_double2(c.x * ir, c.y * ir);
-                    if (!m0) b = b.times(w);
+                    const double f = double(h + LPP * k) * ir;
+                    const double2 b = m0 ? make_double2(0.0, 0.0) : below[32 * k];
+                    st64[32 * (2 * NS + k)] = make_double2(f * b.x, f * b.y);
+                    if (NORM) {
+                        const double2 c = cs[32 * k];
+                        st64[32 * (3 * NS + k)] = make_double2((m0 ? inv_sqrt2 : c.x) * ir, c.y * ir);
+                    }
                 }
-                a = a.times(w);
             }
+            if (LPP > 1) __syncwarp();
+            if (h == 0) cs[0].x = inv_sqrt2;
         }
 
         // A point with a zero coordinate has a zero Qtilde, c_m or s_m at every
