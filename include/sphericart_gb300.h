@@ -149,10 +149,13 @@ typedef enum {
  *                    SLICE: 8, 16 or 32 (0 = by l_max)
  * DEGREE kernels read warps_per_block (0..8, 0 = by shared memory),
  * blocks_per_sm and lanes_per_point (1, 2 or 4 lanes per point for DEGREE, 0 =
- * by measurement, for FP64 arithmetic also by the number of points, up to 8;
- * launch_info reports the least; DEGREE_DOWN takes 1). ROW kernels read
- * warps_per_block (forward 0..2, backward 0..8; 0 = one block of up to 12
- * (backward 16) warps per SM, 2 with Hessians), blocks_per_sm, and lanes_per_point as the forward window policy (0 = by
+ * by measurement, for FP64 arithmetic also by the number of points, up to 8,
+ * and never fewer from l_max 27 than AUTO's for many points, which launch_info
+ * reports; FP64 results do not depend on the lanes; DEGREE_DOWN takes 1). ROW
+ * kernels read warps_per_block (forward 0..2, backward 0..8) and blocks_per_sm:
+ * their product is the number of warps on an SM, in one block as long as they
+ * fit (0 for either: as many as fit, up to 16; with Hessians the blocks are the
+ * caller's, 0 = 2 warps), and lanes_per_point as the forward window policy (0 = by
  * l_max, 1, 2; with Hessians 0/2 = 136 columns, 1 = one degree of l_max,
  * 3 = 256 columns).
  * The POINT default (no shape given and none tuned) fills ~48 KB tiles (FP32,

@@ -533,6 +533,7 @@ int degree_default_lpp(int l_max, int dtype, int qprec) {
 // channels to share out, and none for more than l_max + 1 lanes: FP32 values,
 // l_max 3, 4k points, 5.7/5.3/8.0 us, FP64 gradients, l_max 6, scaled, 10k points
 // 24.7/24.2/-, 4k -/15.0/18.6, 1k -/14.4/13.2.
+constexpr int64_t kManyPoints = int64_t(1) << 40;
 int degree_f64_lpp(int64_t n, int l_max, bool grad, bool mixed) {
     int lpp;
     if (grad) lpp = l_max > 26 ? 8 : (l_max >= (mixed ? 16 : 12) ? 4 : 2);
@@ -841,9 +842,16 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
             set_error("DEGREE_DOWN runs one lane per point (the downward recursion is sequential in m)");
             return SPH_EINVAL;
         }
-        if (lpp == 0)
-            lpp = dtype == SPH_F64 || mixed ? degree_f64_lpp(n, l_max, grad, mixed)
-                                            : degree_default_lpp(l_max, dtype, qprec);
+        if (dtype == SPH_F64 || mixed) {
+            // From l_max 27 the state of a point takes so much shared memory that fewer lanes
+            // than AUTO's leave few warps on an SM (gradients, l_max 50, 100k points, ms at
+            // 1 / 2 / 4 / 8 lanes: 30/12/7.4/5.2): an explicit 1, 2 or 4 is raised. The results
+            // are the same.
+            const int least = l_max > 26 ? degree_f64_lpp(kManyPoints, l_max, grad, mixed) : 1;
+            lpp = lpp == 0 ? degree_f64_lpp(n, l_max, grad, mixed) : std::max(lpp, least);
+        } else if (lpp == 0) {
+            lpp = degree_default_lpp(l_max, dtype, qprec);
+        }
         int e;
         if (fam == SPH_KERNEL_DEGREE_DOWN)
             e = degree_fwd_down(a);

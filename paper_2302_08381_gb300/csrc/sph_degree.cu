@@ -818,18 +818,22 @@ int launch_degree(const FwdArgs& a, const TQ* tb) {
 #if !SPH_DEGREE_DOWN
 // The lane-private state of degree_f64_kernel takes more shared memory than
 // degree_fwd_kernel's columns: a block of the requested warps that does not
-// fit runs fewer, and one lane per point at l_max 128 runs two. What is
-// refused is decided by the size of degree_fwd_kernel's block, as for FP32.
+// fit runs fewer (one always fits: the caller gives at least 4 lanes from l_max 27).
+// What is refused is decided by the size of degree_fwd_kernel's block at the
+// requested lanes, as for FP32.
 template <typename TI, typename TO, bool GRAD, bool NORM>
 int launch_f64(const FwdArgs& a, const double* tb) {
     constexpr int PPW = 32 / kLPP;
     auto kern = degree_f64_kernel<TI, TO, GRAD, NORM, kLPP>;
     const size_t optin = size_t(max_smem_optin());
     const size_t per_warp = f64_warp_bytes<kLPP, TO, GRAD, NORM>(a.l_max);
-    if (a.launch.warps_per_block > 0 &&
-        size_t(a.launch.warps_per_block) * degree_warp_bytes<kLPP, double, TO, GRAD, false>(a.l_max) > optin)
+    const int lanes = a.launch.lanes_per_point > 0 ? a.launch.lanes_per_point : kLPP;  // as requested
+    const size_t checked = lanes == 1   ? degree_warp_bytes<1, double, TO, GRAD, false>(a.l_max)
+                           : lanes == 2 ? degree_warp_bytes<2, double, TO, GRAD, false>(a.l_max)
+                           : lanes == 4 ? degree_warp_bytes<4, double, TO, GRAD, false>(a.l_max)
+                                        : degree_warp_bytes<8, double, TO, GRAD, false>(a.l_max);
+    if (a.launch.warps_per_block > 0 && size_t(a.launch.warps_per_block) * checked > optin)
         return int(cudaErrorInvalidConfiguration);
-    if (kLPP == 1 && per_warp > optin) return degree_fwd_up2(a);
     const int64_t ntiles = (a.n + PPW - 1) / PPW;
     // Few tiles, up to eight per SM, in one-warp blocks: they spread evenly (gradients,
     // scaled, l_max 8, 8k points 28.6 us in blocks of 4 warps, 26.2 so; 16k 51.4, 38.7;
