@@ -91,6 +91,12 @@ typedef enum { SPH_Q_NATIVE = 0, SPH_Q_F64 = 1 } sph_qprec;
  * l_max <= SPH_MAX_L_POINT (except bfloat16 Hessians); else ROW for FP32
  * arithmetic up to l_max 63; else DEGREE for bfloat16 storage without
  * Hessians; else SLICE.
+ * Families differ in the last bits. Where the choice goes by the number of
+ * points (SPH_F64 values of l_max 11..13 and gradients of 5..8, mixed mode of
+ * l_max 3 and 4, normalized FP32 Hessians of 14 and 15), so do the results of
+ * one point in calls of different size, as of a set in one call and split over
+ * GPUs; name the family to have them equal. sphericart_compute_host chooses by
+ * the whole call. Launch shapes and lanes per point do not change results.
  *   POINT:  one thread per point, the whole (l, m) recursion unrolled in
  *           registers for a compile-time l_max, outputs staged in shared memory
  *           and written with bulk (TMA) copies.
@@ -209,7 +215,8 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
  * for its end; the call itself returns without synchronising. Host buffers
  * should be pinned (cudaHostAlloc / cudaHostRegister) for the copies to be
  * asynchronous. Layouts, dtype and out as in sphericart_compute_ex (FP32 or
- * FP64, optional bf16 store); no Hessians. Errors: SPH_EINVAL for bad sizes,
+ * FP64, optional bf16 store); no Hessians. The results are those of one
+ * sphericart_compute_ex call on all points. Errors: SPH_EINVAL for bad sizes,
  * NULL pointers or a workspace too small for two 32-point stages. */
 int sphericart_compute_host(const void* xyz_host, int64_t n, int l_max, int normalized,
                             int dtype, int out, void* sph_host, void* dsph_host,

@@ -645,36 +645,10 @@ int ensure_device(const char* what) {
 
 }  // namespace sph
 
-using namespace sph;
+namespace sph {
 
-extern "C" {
-
-int sphericart_version(void) { return 10000; }
-
-const char* sphericart_last_error(void) { return last_error_message(); }
-
-int sphericart_max_l(int dtype, int qprec, int kernel) {
-    if (kernel == SPH_KERNEL_POINT) return (qprec == SPH_Q_F64 && dtype == SPH_F32) ? -1 : SPH_MAX_L_POINT;
-    if (kernel == SPH_KERNEL_POINT_HC) return (qprec == SPH_Q_F64 && dtype == SPH_F32) ? -1 : kHcMaxL;
-    if (kernel == SPH_KERNEL_ROW) return (dtype == SPH_F32 && qprec == SPH_Q_NATIVE) ? kRowMaxL : -1;
-    (void)dtype;
-    return SPH_MAX_L;
-}
-
-int sphericart_host_table(int l_max, int which, double* out) {
-    if (!out || l_max < 0 || l_max > SPH_MAX_L || which < 0 || which > 8) {
-        set_error("host_table: bad arguments (l_max=%d which=%d)", l_max, which);
-        return SPH_EINVAL;
-    }
-    const HostTables& h = host_tables();
-    const std::vector<double>* src[] = {&h.F, &h.qll, &h.a, &h.b, &h.e, &h.fz, &h.d, &h.al, &h.be};
-    std::memcpy(out, src[which]->data(), sizeof(double) * size_t(tri_size(l_max)));
-    return SPH_OK;
-}
-
-int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized, int dtype, int out, int qprec,
-                          int kernel, const sph_launch* launch, void* sph, void* dsph, void* ddsph,
-                          void* stream) {
+int compute_routed(const void* xyz, int64_t n, int l_max, int normalized, int dtype, int out, int qprec, int kernel,
+                   const sph_launch* launch, void* sph, void* dsph, void* ddsph, void* stream, int64_t n_call) {
     int st = check_common(n, l_max, dtype, kernel);
     if (st) return st;
     if (out != SPH_OUT_SAME && out != SPH_OUT_BF16) {
@@ -698,8 +672,8 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
     int fam = kernel;
     const bool hess_bf16 = ddsph && out == SPH_OUT_BF16;
     if (fam == SPH_KERNEL_AUTO)
-        fam = auto_family(l_max, dtype, out, qprec, ddsph != nullptr, dsph != nullptr, normalized, n);
-    if (kernel == SPH_KERNEL_AUTO && !launch && dtype == SPH_F64 && !ddsph && f64_prefers_degree(n, l_max, grad, normalized)) {
+        fam = auto_family(l_max, dtype, out, qprec, ddsph != nullptr, dsph != nullptr, normalized, n_call);
+    if (kernel == SPH_KERNEL_AUTO && !launch && dtype == SPH_F64 && !ddsph && f64_prefers_degree(n_call, l_max, grad, normalized)) {
         // POINT needs no device tables: a call captured before any upload stays there
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (device_tables_f64_ready() ||
@@ -711,7 +685,7 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
     }
     int hc = 0;
     const bool mixed_point = kernel == SPH_KERNEL_AUTO && !launch && mixed && !ddsph && out == SPH_OUT_SAME &&
-                             mixed_prefers_point(n, l_max);
+                             mixed_prefers_point(n_call, l_max);
     if (mixed_point) {
         fam = SPH_KERNEL_POINT;
         hc = 1;
@@ -775,7 +749,7 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
             a.launch.blocks_per_sm == 0 && a.launch.lanes_per_point == 0) {
             if (point4_default(l_max, grad, eo, hess, hc, normalized))
                 a.launch.lanes_per_point = 4;
-            else if (point10_default(l_max, hess, normalized, dtype, out, n))
+            else if (point10_default(l_max, hess, normalized, dtype, out, n_call))
                 a.launch.lanes_per_point = 10;
         }
         const int lpp = a.launch.lanes_per_point;
@@ -885,6 +859,41 @@ int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized,
     }
     if (!valid_lanes(a.launch)) return SPH_EINVAL;
     return cuda_status(slice_fwd(a), "SLICE forward launch");
+}
+
+}  // namespace sph
+
+using namespace sph;
+
+extern "C" {
+
+int sphericart_version(void) { return 10000; }
+
+const char* sphericart_last_error(void) { return last_error_message(); }
+
+int sphericart_max_l(int dtype, int qprec, int kernel) {
+    if (kernel == SPH_KERNEL_POINT) return (qprec == SPH_Q_F64 && dtype == SPH_F32) ? -1 : SPH_MAX_L_POINT;
+    if (kernel == SPH_KERNEL_POINT_HC) return (qprec == SPH_Q_F64 && dtype == SPH_F32) ? -1 : kHcMaxL;
+    if (kernel == SPH_KERNEL_ROW) return (dtype == SPH_F32 && qprec == SPH_Q_NATIVE) ? kRowMaxL : -1;
+    (void)dtype;
+    return SPH_MAX_L;
+}
+
+int sphericart_host_table(int l_max, int which, double* out) {
+    if (!out || l_max < 0 || l_max > SPH_MAX_L || which < 0 || which > 8) {
+        set_error("host_table: bad arguments (l_max=%d which=%d)", l_max, which);
+        return SPH_EINVAL;
+    }
+    const HostTables& h = host_tables();
+    const std::vector<double>* src[] = {&h.F, &h.qll, &h.a, &h.b, &h.e, &h.fz, &h.d, &h.al, &h.be};
+    std::memcpy(out, src[which]->data(), sizeof(double) * size_t(tri_size(l_max)));
+    return SPH_OK;
+}
+
+int sphericart_compute_ex(const void* xyz, int64_t n, int l_max, int normalized, int dtype, int out, int qprec,
+                          int kernel, const sph_launch* launch, void* sph, void* dsph, void* ddsph,
+                          void* stream) {
+    return compute_routed(xyz, n, l_max, normalized, dtype, out, qprec, kernel, launch, sph, dsph, ddsph, stream, n);
 }
 
 int sphericart_compute(const float* xyz, int64_t n, int l_max, int normalized, float* sph, float* dsph,

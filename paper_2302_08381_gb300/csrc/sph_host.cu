@@ -122,8 +122,8 @@ extern "C" int sphericart_compute_host(const void* xyz_host, int64_t n, int l_ma
         if (e == cudaSuccess) e = cudaEventRecord(P->h2d_ev[b], P->h2d);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(P->comp, P->h2d_ev[b], 0);
         if (e == cudaSuccess) {
-            const int stt = sphericart_compute_ex(dx, cnt, l_max, normalized, dtype, out, SPH_Q_NATIVE,
-                                                  SPH_KERNEL_AUTO, nullptr, ds, dd, nullptr, P->comp);
+            const int stt = compute_routed(dx, cnt, l_max, normalized, dtype, out, SPH_Q_NATIVE, SPH_KERNEL_AUTO,
+                                           nullptr, ds, dd, nullptr, P->comp, n);
             if (stt != SPH_OK) return stt;  // message already set
         }
         if (e == cudaSuccess) e = cudaEventRecord(P->comp_ev[b], P->comp);

@@ -212,6 +212,11 @@ int degree_fwd_up4(const FwdArgs& a);
 int degree_fwd_up8(const FwdArgs& a);  // FP64 arithmetic only
 int degree_fwd_down(const FwdArgs& a);
 
+// sphericart_compute_ex on part of a call: AUTO's kernel is chosen by the whole
+// call's n_call points, so that its parts have the bits of the whole.
+int compute_routed(const void* xyz, int64_t n, int l_max, int normalized, int dtype, int out, int qprec, int kernel,
+                   const sph_launch* launch, void* sph, void* dsph, void* ddsph, void* stream, int64_t n_call);
+
 // ROW kernels (FP32 arithmetic, 16 <= l_max <= 63, values and gradients):
 // part 0 covers 3..5 channels per lane (l_max <= 47), part 1 6..8.
 int row_fwd_part0(const FwdArgs& a);
