@@ -850,7 +850,9 @@ def run_variants_leg(torch, api, inputs, dev, stream, flush):
         # headline does); value-only / gradient / bf16 / FP64 shapes are tuned
         # separately, Hessian shapes keep their defaults; the other families
         # take their default shapes.
-        auto_point = L <= 16 if dt == torch.float32 else L <= 11  # where AUTO runs the POINT kernels
+        # where AUTO runs the POINT kernels (FP64: or, by the number of points, DEGREE,
+        # which the autotuner then compares with)
+        auto_point = L <= (16 if dt == torch.float32 else 8 if kw.get("gradients") else 13)
         if auto_point and "kernel" not in kw and "qprec" not in kw and not kw.get("hessians"):
             from paper_2302_08381_gb300 import _capi as C
 

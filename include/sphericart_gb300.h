@@ -465,7 +465,8 @@ int sphericart_launch_info(int l_max, int dtype, int out, int grad, int hess,
 /* sphericart_set_launch: installs a tuned launch shape for forward calls with
  * this (l_max, dtype, out, grad) on the current device; used by AUTO/POINT
  * calls that pass launch == NULL (grad: 0 values, 1 + gradients, 2 + gradients
- * and Hessians). points_per_tile etc. are validated; lanes_per_point 0, 1, 4
+ * and Hessians). With a shape installed AUTO stays on POINT where it would
+ * choose DEGREE by the number of points. points_per_tile etc. are validated; lanes_per_point 0, 1, 4
  * (FP32 gradients), 10 or 16 (FP32 Hessians, FP32 storage). */
 int sphericart_set_launch(int l_max, int dtype, int out, int grad,
                           const sph_launch* launch);
@@ -480,7 +481,9 @@ int sphericart_tune_clear(void);
  * buffers (sph/dsph are overwritten), `reps` timed runs each (median, CUDA
  * events on `stream`; synchronises), installs the fastest for later calls
  * with launch == NULL (as sphericart_set_launch) and returns it in *best
- * (and its time in *best_ms if non-NULL). l_max <= SPH_MAX_L_POINT, n > 0.
+ * (and its time in *best_ms if non-NULL). Where AUTO runs this many SPH_F64
+ * points on DEGREE, and DEGREE is faster than every shape, none is installed
+ * (an installed one is removed) and *best is {0, 0, 0, 0}. l_max <= SPH_MAX_L_POINT, n > 0.
  * The autotuner and the batch autotuner are the project's own: the paper
  * grows its shared-memory allocation on first call instead (Section 3). */
 int sphericart_autotune(const void* xyz, int64_t n, int l_max, int normalized,

@@ -484,6 +484,13 @@ sph_launch point_fwd_shape(int L, int grad) {
     return s;
 }
 
+void tuned_remove(int L, int dtype, int out, int grad) {
+    int d = -1;
+    if (cudaGetDevice(&d) != cudaSuccess) return;
+    std::lock_guard<std::mutex> lk(g_mu);
+    g_tuned.erase(TuneKey{d, L, dtype, out, grad});
+}
+
 bool tuned_launch(int L, int dtype, int out, int grad, sph_launch* s) {
     int d = -1;
     if (cudaGetDevice(&d) != cudaSuccess) {
@@ -562,6 +569,8 @@ namespace {
 // a point over lanes from l_max 3.
 bool mixed_prefers_point(int64_t n, int l_max) { return l_max <= kMixedHcMaxL && (l_max <= 2 || n >= 8192); }
 
+}  // namespace
+
 // FP64 requests below auto_family's DEGREE limits that run faster there all
 // the same, by the number of points. Measured on GB300, us, POINT / DEGREE.
 // Gradients, scaled: l_max 5 1k points 14.2/11.9, 4k 14.2/12.8, 8k 14.1/15.1; 6 4k
@@ -570,12 +579,15 @@ bool mixed_prefers_point(int64_t n, int l_max) { return l_max <= kMixedHcMaxL &&
 // 29.1/26.2, 16k 56/39, 100k 223/197. Normalized: 5 8k 23.0/18.2, 100k 116/119; 6 8k
 // 29.2/21.0; 7 10k 39/31, 100k 272/177. Values: 11 32k 46/40, 100k 100/90; 12 16k
 // 26.2/27.6, 32k 49/46; 13 16k 29.8/30.8, 100k 174/128; 10 100k 78/79.
-bool f64_prefers_degree(int64_t n, int l_max, bool grad, bool normalized) {
+bool f64_prefers_degree(int64_t n, int l_max, int dtype, bool grad, bool normalized) {
+    if (dtype != SPH_F64) return false;
     if (!grad) return n >= 32768 && l_max >= 11;
     if (n < 256) return false;
     if (l_max >= 7) return normalized || n <= 8192 || n > 12288;
     return l_max >= 5 && n <= (normalized ? 8192 : 4096);
 }
+
+namespace {
 
 // AUTO kernel family of a forward request (measured on GB300). POINT
 // (compile-time l_max, TMA bulk stores) wins whenever it applies in FP32, and
@@ -673,7 +685,9 @@ int compute_routed(const void* xyz, int64_t n, int l_max, int normalized, int dt
     const bool hess_bf16 = ddsph && out == SPH_OUT_BF16;
     if (fam == SPH_KERNEL_AUTO)
         fam = auto_family(l_max, dtype, out, qprec, ddsph != nullptr, dsph != nullptr, normalized, n_call);
-    if (kernel == SPH_KERNEL_AUTO && !launch && dtype == SPH_F64 && !ddsph && f64_prefers_degree(n_call, l_max, grad, normalized)) {
+    sph_launch installed;
+    if (kernel == SPH_KERNEL_AUTO && !launch && !ddsph && f64_prefers_degree(n_call, l_max, dtype, grad, normalized) &&
+        !tuned_launch(l_max, dtype, out, grad, &installed)) {  // an installed shape is a POINT shape
         // POINT needs no device tables: a call captured before any upload stays there
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (device_tables_f64_ready() ||

@@ -155,6 +155,9 @@ constexpr int kMixedHcMaxL = 4;
 // Whether AUTO runs the hybrid instead of the all-recursion POINT forward
 // (values, or values and gradients; no Hessians).
 bool point_hybrid_wins(int l_max, int dtype, bool grad);
+// Whether AUTO, with no installed shape, runs an FP64 request that POINT takes on
+// DEGREE, by the number of points.
+bool f64_prefers_degree(int64_t n, int l_max, int dtype, bool grad, bool normalized);
 
 struct BwdArgs {
     const void* xyz;
@@ -194,6 +197,7 @@ BatchOneFn batch_one_fn(int gn);
 // Tuned POINT forward shape installed for (l_max, dtype, out, grad) on the
 // current device; false if none.
 bool tuned_launch(int L, int dtype, int out, int grad, sph_launch* s);
+void tuned_remove(int L, int dtype, int out, int grad);
 
 // The POINT forward launch shape for FP32 values (+ gradients when grad) at
 // this l_max on the current device: the tuned one if installed, else the

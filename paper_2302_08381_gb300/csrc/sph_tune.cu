@@ -158,6 +158,24 @@ int sphericart_autotune(const void* xyz, int64_t n, int l_max, int normalized, i
     // one lane per point (lanes_per_point 1), then, for FP32 arithmetic with
     // gradients, one lane per output plane (lanes_per_point 4, <= 8 points)
     const bool four = grad && dtype == SPH_F32 && fam == SPH_KERNEL_POINT;
+    auto median = [&](int family, const sph_launch* s) -> float {  // ms of `reps` runs, -1 on an error
+        std::vector<float> ts;
+        for (int r = 0; r < reps; ++r) {
+            cudaEventRecord(ev.a, st);
+            sphericart_compute_ex(xyz, n, l_max, normalized, dtype, out, SPH_Q_NATIVE, family, s, sph, dsph, nullptr,
+                                  stream);
+            cudaEventRecord(ev.b, st);
+            if (cudaEventSynchronize(ev.b) != cudaSuccess) {
+                set_error("autotune: %s", cudaGetErrorString(cudaGetLastError()));
+                return -1.f;
+            }
+            float ms = 0.f;
+            cudaEventElapsedTime(&ms, ev.a, ev.b);
+            ts.push_back(ms);
+        }
+        std::sort(ts.begin(), ts.end());
+        return ts[ts.size() / 2];
+    };
     for (int pass = 0; pass < (four ? 2 : 1); ++pass)
     for (int P : Ps) {
         if (P % mult != 0 || (pass == 1 && P > 8)) continue;
@@ -172,22 +190,8 @@ int sphericart_autotune(const void* xyz, int64_t n, int l_max, int normalized, i
                     cudaGetLastError();
                     continue;  // shape not launchable here (occupancy, limits)
                 }
-                std::vector<float> ts;
-                for (int r = 0; r < reps; ++r) {
-                    cudaEventRecord(ev.a, st);
-                    sphericart_compute_ex(xyz, n, l_max, normalized, dtype, out, SPH_Q_NATIVE, fam, &s, sph, dsph,
-                                          nullptr, stream);
-                    cudaEventRecord(ev.b, st);
-                    if (cudaEventSynchronize(ev.b) != cudaSuccess) {
-                        set_error("autotune: %s", cudaGetErrorString(cudaGetLastError()));
-                        return SPH_ECUDA;
-                    }
-                    float ms = 0.f;
-                    cudaEventElapsedTime(&ms, ev.a, ev.b);
-                    ts.push_back(ms);
-                }
-                std::sort(ts.begin(), ts.end());
-                const float t = ts[ts.size() / 2];
+                const float t = median(fam, &s);
+                if (t < 0.f) return SPH_ECUDA;
                 if (t < best_t) {
                     best_t = t;
                     best_s = s;
@@ -198,6 +202,19 @@ int sphericart_autotune(const void* xyz, int64_t n, int l_max, int normalized, i
     if (best_s.points_per_tile == 0) {
         set_error("autotune: no launchable shape");
         return SPH_EUNSUPPORTED;
+    }
+    if (f64_prefers_degree(n, l_max, dtype, grad != 0, normalized != 0) &&
+        sphericart_compute_ex(xyz, n, l_max, normalized, dtype, out, SPH_Q_NATIVE, SPH_KERNEL_DEGREE, nullptr, sph,
+                              dsph, nullptr, stream) == SPH_OK) {
+        // with no shape installed AUTO runs DEGREE here: that stays so where it is the faster
+        const float t = median(SPH_KERNEL_DEGREE, nullptr);
+        if (t < 0.f) return SPH_ECUDA;
+        if (t <= best_t) {
+            tuned_remove(l_max, dtype, out, grad);
+            *best = sph_launch{0, 0, 0, 0};
+            if (best_ms) *best_ms = t;
+            return SPH_OK;
+        }
     }
     *best = best_s;
     if (best_ms) *best_ms = best_t;
