@@ -70,6 +70,30 @@ int max_smem_optin() {
 
 namespace {
 
+// `bytes` of host data in new device memory, nullptr (message set) on an error. Made
+// in relaxed capture mode and copied on a stream of its own: a graph capture that
+// another stream or thread has going on, which forbids cudaMalloc and the legacy
+// stream to every thread, is not disturbed by a first call that needs tables.
+void* upload(const void* host, size_t bytes) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    void* p = nullptr;
+    cudaStream_t st = nullptr;
+    cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(p, host, bytes, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (st) cudaStreamDestroy(st);
+    if (e != cudaSuccess) {
+        if (p) cudaFree(p);
+        p = nullptr;
+        cudaGetLastError();
+        set_error("upload of %zu bytes of device tables: %s", bytes, cudaGetErrorString(e));
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return p;
+}
+
 // Uploads kSliceTables values per (l, m) entry, produced by `pack`, as FP32 or
 // FP64 into `slot` (once per device).
 template <typename Pack>
@@ -91,17 +115,7 @@ const void* upload_packed(void*& slot, int dtype, Pack pack) {
                     reinterpret_cast<float*>(host.data())[o] = static_cast<float>(v[t]);
             }
         }
-    void* p = nullptr;
-    if (cudaMalloc(&p, host.size()) != cudaSuccess) {
-        set_error("cudaMalloc of %zu bytes for device tables failed", host.size());
-        return nullptr;
-    }
-    if (cudaMemcpy(p, host.data(), host.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
-        cudaFree(p);
-        set_error("upload of device tables failed");
-        return nullptr;
-    }
-    slot = p;
+    slot = upload(host.data(), host.size());
     return slot;
 }
 
@@ -232,20 +246,8 @@ const void* device_row_tables() {
                 g4[4 * o + 1] = float(h.g3[i] * unfold);
                 g4[4 * o + 2] = float(h.g4[i] * unfold);
             }
-    void* p = nullptr;
-    if (cudaMalloc(&p, host.size() * sizeof(float)) != cudaSuccess) {
-        cudaGetLastError();
-        set_error("cudaMalloc of the ROW tables failed");
-        return nullptr;
-    }
-    if (cudaMemcpy(p, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(p);
-        set_error("upload of the ROW tables failed");
-        return nullptr;
-    }
-    slots[d] = p;
-    return p;
+    slots[d] = upload(host.data(), host.size() * sizeof(float));
+    return slots[d];
 }
 
 uint32_t* device_status_word() {
@@ -688,11 +690,12 @@ int compute_routed(const void* xyz, int64_t n, int l_max, int normalized, int dt
     sph_launch installed;
     if (kernel == SPH_KERNEL_AUTO && !launch && !ddsph && f64_prefers_degree(n_call, l_max, dtype, grad, normalized) &&
         !tuned_launch(l_max, dtype, out, grad, &installed)) {  // an installed shape is a POINT shape
-        // POINT needs no device tables: a call captured before any upload stays there
+        // POINT needs no device tables: a call captured before any upload stays
+        // there, and so does one whose upload fails
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (device_tables_f64_ready() ||
             (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) == cudaSuccess &&
-             cap == cudaStreamCaptureStatusNone))
+             cap == cudaStreamCaptureStatusNone && device_tables_f64()))
             fam = SPH_KERNEL_DEGREE;
         else
             cudaGetLastError();
