@@ -500,9 +500,14 @@ __device__ __forceinline__ bool f64_step(int l, int m, const double4_32a& t, dou
                                          double ly, double lz, const double2& q, double qr, const double2& c,
                                          const double2& ci, const double2& c1, F64Step& o) {
     bool in = true;
-    // a * b, or 0 where it is not `used`
-    auto mul = [&](double a, const Mul64& b, bool used) {
-        if constexpr (MUL == Mul::kFp64) return used ? a * b.v : 0.0;
+    // a * b, or 0 where it is not `used`; `other` is then the factor that is not zero by
+    // its place, and where it is infinite or NaN (on the FP64 pipe: no such operand
+    // is in the other's range) so is the product
+    auto mul = [&](double a, const Mul64& b, bool used, double other = 0.0) {
+        if constexpr (MUL == Mul::kFp64) {
+            const bool nan = (uint32_t(__double2hiint(other)) & 0x7ff00000u) == 0x7ff00000u;
+            return used ? a * b.v : (nan ? __hiloint2double(0x7ff80000, 0) : 0.0);
+        }
         bool ok = b.ok;
         const double p = b.template fast<MUL == Mul::kIntZero>(a, ok);
         in = in && (ok || !used);
@@ -521,21 +526,21 @@ __device__ __forceinline__ bool f64_step(int l, int m, const double4_32a& t, dou
     if (GRAD) {
         const double E1 = mul(qr, Mul64(e), m < l - 1);  // e Qtilde_{l-1}^{m+1}
         const Mul64 E(E1);
-        double X = mul(P.x, E, m < l - 1), Y = mul(P.y, E, m < l - 1), Z = mul(q.x, Mul64(t.w), m < l);
+        double X = mul(P.x, E, m < l - 1, P.x), Y = mul(P.y, E, m < l - 1, P.y), Z = mul(q.x, Mul64(t.w), m < l);
         if (NORM) {
             X = fma(-lx, o.q, X);
             Y = fma(-ly, o.q, Y);
             Z = fma(-lz, o.q, Z);
         }
-        const double tc = mul(c1.x, Q, m1), ts = mul(c1.y, Q, m > 1);
+        const double tc = mul(c1.x, Q, m1), ts = mul(c1.y, Q, m > 1, m1 ? o.q : 0.0);
         o.xc = fma(X, ci.x, tc);
         o.xs = fma(X, ci.y, ts);
         o.yc = fma(Y, ci.x, -ts);
         o.ys = fma(Y, ci.y, tc);
         const Mul64 Zm(Z);
         const bool zu = NORM ? l > 0 : m < l;
-        o.zc = mul(ci.x, Zm, zu);
-        o.zs = mul(ci.y, Zm, zu && m1);
+        o.zc = mul(ci.x, Zm, zu, NORM ? Z : ci.x);
+        o.zs = mul(ci.y, Zm, zu && m1, NORM ? Z : ci.y);
     }
     return in;
 }
