@@ -161,7 +161,7 @@ typedef enum {
  * kernels read warps_per_block (forward 0..2, backward 0..8) and blocks_per_sm:
  * their product is the number of warps on an SM, in one block as long as they
  * fit (0 for either: as many as fit, up to 16; with Hessians the blocks are the
- * caller's, 0 = 2 warps), and lanes_per_point as the forward window policy (0 = by
+ * caller's, 0..2, 0 = 1 warp, from l_max 40 2), and lanes_per_point as the forward window policy (0 = by
  * l_max, 1, 2; with Hessians 0/2 = 136 columns, 1 = one degree of l_max,
  * 3 = 256 columns).
  * The POINT default (no shape given and none tuned) fills ~48 KB tiles (FP32,
@@ -458,7 +458,9 @@ int sphericart_device_status(uint32_t* status);
 
 /* sphericart_launch_info: the launch shape the library would use for a
  * forward call (after tuning), for inspection. kernel_out receives the
- * family (POINT or SLICE). Host-only except for a device-properties query. */
+ * family; lanes_per_point is that of the kernel (ROW 8, DEGREE the number for
+ * many points), and a zero is left to the call. Host-only except for a
+ * device-properties query. */
 int sphericart_launch_info(int l_max, int dtype, int out, int grad, int hess,
                            int* kernel_out, sph_launch* launch_out);
 

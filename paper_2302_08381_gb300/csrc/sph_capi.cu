@@ -522,13 +522,9 @@ bool valid_lanes(const sph_launch& s) {
 
 bool aligned(const void* p, size_t a) { return reinterpret_cast<uintptr_t>(p) % a == 0; }
 
-// Lanes per point of the upward DEGREE kernel when the caller leaves it 0:
-// FP32 arithmetic 4; FP64 arithmetic at least these, see degree_f64_lpp.
-int degree_default_lpp(int l_max, int dtype, int qprec) {
-    if (dtype == SPH_F64) return l_max >= 24 ? 4 : (l_max >= 10 ? 2 : 1);
-    if (qprec == SPH_Q_F64) return 2;
-    return 4;
-}
+// Lanes per point of the upward DEGREE kernel with FP32 arithmetic when the caller
+// leaves it 0.
+constexpr int kDegreeF32Lanes = 4;
 
 // FP64 arithmetic (degree_f64_kernel). A point's lane-private state grows with
 // l_max, and with few warps on an SM the latency of the integer products shows:
@@ -841,7 +837,7 @@ int compute_routed(const void* xyz, int64_t n, int l_max, int normalized, int dt
             const int least = l_max > 26 ? degree_f64_lpp(kManyPoints, l_max, grad, mixed) : 1;
             lpp = lpp == 0 ? degree_f64_lpp(n, l_max, grad, mixed) : std::max(lpp, least);
         } else if (lpp == 0) {
-            lpp = degree_default_lpp(l_max, dtype, qprec);
+            lpp = kDegreeF32Lanes;
         }
         int e;
         if (fam == SPH_KERNEL_DEGREE_DOWN)
@@ -1045,10 +1041,12 @@ int sphericart_launch_info(int l_max, int dtype, int out, int grad, int hess, in
     if (hc) fam = SPH_KERNEL_POINT;  // same launch shapes
     if (fam == SPH_KERNEL_DEGREE) {
         *kernel_out = SPH_KERNEL_DEGREE;
-        *launch_out = sph_launch{0, 0, 0, degree_default_lpp(l_max, dtype, SPH_Q_NATIVE)};
+        *launch_out = sph_launch{
+            0, 0, 0, dtype == SPH_F64 ? degree_f64_lpp(kManyPoints, l_max, grad != 0, false) : kDegreeF32Lanes};
     } else if (fam == SPH_KERNEL_ROW) {
         *kernel_out = SPH_KERNEL_ROW;
-        *launch_out = sph_launch{0, 1, 0, 8};
+        // (0 warps: as many as fit; Hessians: as launch_row_hess)
+        *launch_out = sph_launch{0, hess ? (l_max < 40 ? 1 : 2) : 0, 0, 8};
     } else if (fam == SPH_KERNEL_POINT) {
         *kernel_out = hc ? SPH_KERNEL_POINT_HC : SPH_KERNEL_POINT;
         sph_launch s{0, 0, 0, 0};
