@@ -79,7 +79,7 @@ typedef enum { SPH_Q_NATIVE = 0, SPH_Q_F64 = 1 } sph_qprec;
 
 /* Kernel family. AUTO picks, by measurement on GB300: DEGREE for FP64
  * arithmetic without Hessians (the mixed mode, except with FP32 storage to
- * l_max 4, from l_max 3 on 8,192 points or more: POINT_HC with FP64
+ * l_max 4, gradients from l_max 3 on 8,192 points or more: POINT_HC with FP64
  * arithmetic; SPH_F64 from l_max 14, with
  * gradients from l_max 9, and by the number of points from l_max 11, with
  * gradients 5: launch_info, which takes none, reports the choice for few
@@ -92,8 +92,8 @@ typedef enum { SPH_Q_NATIVE = 0, SPH_Q_F64 = 1 } sph_qprec;
  * arithmetic up to l_max 63; else DEGREE for bfloat16 storage without
  * Hessians; else SLICE.
  * Families differ in the last bits. Where the choice goes by the number of
- * points (SPH_F64 values of l_max 11..13 and gradients of 5..8, mixed mode of
- * l_max 3 and 4, normalized FP32 Hessians of 14 and 15), so do the results of
+ * points (SPH_F64 values of l_max 11..13 and gradients of 5..8, mixed-mode
+ * gradients of 3 and 4, normalized FP32 Hessians of 14 and 15), so do the results of
  * one point in calls of different size, as of a set in one call and split over
  * GPUs; name the family to have them equal. sphericart_compute_host chooses by
  * the whole call. Launch shapes and lanes per point do not change results.

@@ -407,13 +407,16 @@ bool point4_default(int L, int grad, int elem, int hess, int hc, int normalized)
 // Whole 32-point tiles (the recursion runs on full warps). Small tiles in blocks
 // of two warps on a grid of 32 blocks per SM scheduled in waves (fused backward,
 // l_max 6: 11 % above a persistent one-wave grid; double backward, waves against
-// one wave, l_max 4 150 / 162 us, 8 324 / 350), except for the double backward
-// with even K (l_max 7 345 / 320) or three buffers of more than 12 KB (6 283 /
-// 257); larger tiles, and few of them, one warp per block and one wave.
+// one wave, l_max 4 151 / 175 us, 8 324 / 350), except for the double backward
+// with even K (l_max 7 345 / 320) or, in FP32, three buffers of more than 12 KB: of
+// the l_max with three buffers that is 6 alone (18.8 KB; 4M points 291 / 267, 400k
+// 40 / 34; l_max 4 has 9.6 KB). In FP64, bound by its pipe, l_max 4 has that size
+// and gains nothing (1M points 713 / 728). Larger tiles, and few of them, one warp
+// per block and one wave.
 sph_launch default_point_bwd(int L, int elem, int dbw, int64_t n) {
     const size_t K = size_t(L + 1) * (L + 1);
     const size_t row = (K % 2 == 0 ? K * elem + 16 : K * elem), tile = 32 * row;
-    const bool wave = dbw && (K % 2 == 0 || (3 * tile > 12 * 1024 && 3 * tile <= 21 * 1024));
+    const bool wave = dbw && (K % 2 == 0 || (elem == 4 && 3 * tile > 12 * 1024 && 3 * tile <= 21 * 1024));
     if (2 * tile <= 24 * 1024 && n >= 128 * int64_t(sm_count())) return sph_launch{32, 2, wave ? 0 : 32, 0};
     return sph_launch{32, 1, 0, 0};
 }
@@ -563,9 +566,13 @@ namespace {
 // whole rows by bulk copies, against DEGREE's stage of a few degrees (400k
 // points, gradients, us: l_max 1 89 on DEGREE, 17 for POINT_HC in FP64; 2 140 /
 // 27; 3 189 / 70; 4 275 / 136; 5 357 / 240, but the conversions of the outputs run
-// on the FP64 pipe in POINT, 144 per point there). Few points: DEGREE's split of
-// a point over lanes from l_max 3.
-bool mixed_prefers_point(int64_t n, int l_max) { return l_max <= kMixedHcMaxL && (l_max <= 2 || n >= 8192); }
+// on the FP64 pipe in POINT, 144 per point there). Gradients of l_max 3 and 4 at few
+// points: DEGREE's split of a point over lanes (3: 4k points 9.0 / 11.5, 8k 12.1 /
+// 11.7; 4: 11.8 / 17.0, 15.4 / 17.3, 10k 19 / 17.3); values stay on POINT_HC (3, 4k
+// points: 6.0 / 4.7; 4: 7.4 / 6.4).
+bool mixed_prefers_point(int64_t n, int l_max, bool grad) {
+    return l_max <= kMixedHcMaxL && (l_max <= 2 || !grad || n >= 8192);
+}
 
 }  // namespace
 
@@ -589,16 +596,17 @@ namespace {
 
 // AUTO kernel family of a forward request (measured on GB300). POINT
 // (compile-time l_max, TMA bulk stores) wins whenever it applies in FP32, and
-// in FP64 up to l_max ~ 10; beyond that FP64 arithmetic (FP64 inputs or the
-// mixed mode) is bound by GB300's FP64 pipe, where the DEGREE family (no idle
-// lanes) is fastest; beyond POINT's range FP32 arithmetic runs on ROW up to
+// in FP64 at small l_max; beyond that FP64 arithmetic (FP64 inputs or the
+// mixed mode) is bound by GB300's FP64 pipe, where the DEGREE family (fewer FP64
+// instructions, no idle lanes) is fastest; beyond POINT's range FP32 arithmetic runs on ROW up to
 // its l_max 63 (1.8-2.2x SLICE; FP32 Hessians 1.2-1.7x), then on SLICE
 // (DEGREE for bf16 storage).
 int auto_family(int l_max, int dtype, int out, int qprec, bool hess, bool grad, int normalized, int64_t n) {
     const bool mixed = dtype == SPH_F32 && qprec == SPH_Q_F64;
-    // FP64: DEGREE with gradients from l_max 9 (measured at 1M-4M points:
-    // l_max 10 / 11 at 1.65x / 2.0x POINT), values from l_max 14 (POINT 8 %
-    // faster at l_max 12, equal at 13; at 10k points POINT up to 16)
+    // FP64 whatever the number of points (POINT / DEGREE, us): gradients from l_max 9
+    // (10: 1k points 43/22, 10k 86/44, 100k 557/269), values from 14 (14: 1k 28.6/15.7,
+    // 10k 30.4/27.1, 100k 203/145; 16: 36/19, 39/34, 259/199). f64_prefers_degree has
+    // the rest.
     if (!hess && (mixed || (dtype == SPH_F64 && (l_max >= 14 || (grad && l_max >= 9))))) return SPH_KERNEL_DEGREE;
     if (!hess && point_hybrid_wins(l_max, dtype, grad)) return SPH_KERNEL_POINT_HC;
     // FP32 Hessians: ROW from row_hess_min_auto (normalized) or beyond POINT's range
@@ -698,7 +706,7 @@ int compute_routed(const void* xyz, int64_t n, int l_max, int normalized, int dt
     }
     int hc = 0;
     const bool mixed_point = kernel == SPH_KERNEL_AUTO && !launch && mixed && !ddsph && out == SPH_OUT_SAME &&
-                             mixed_prefers_point(n_call, l_max);
+                             mixed_prefers_point(n_call, l_max, grad);
     if (mixed_point) {
         fam = SPH_KERNEL_POINT;
         hc = 1;
