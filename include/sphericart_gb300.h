@@ -79,8 +79,8 @@ typedef enum { SPH_Q_NATIVE = 0, SPH_Q_F64 = 1 } sph_qprec;
 
 /* Kernel family. AUTO picks, by measurement on GB300: DEGREE for FP64
  * arithmetic without Hessians (the mixed mode, except with FP32 storage to
- * l_max 4, gradients from l_max 3 on 8,192 points or more: POINT_HC with FP64
- * arithmetic; SPH_F64 from l_max 14, with
+ * l_max 4, gradients from l_max 3 on 8,192 points or more, normalized of 4 below
+ * 65,536: POINT_HC with FP64 arithmetic; SPH_F64 from l_max 14, with
  * gradients from l_max 9, and by the number of points from l_max 11, with
  * gradients 5: launch_info, which takes none, reports the choice for few
  * points); else
@@ -96,7 +96,8 @@ typedef enum { SPH_Q_NATIVE = 0, SPH_Q_F64 = 1 } sph_qprec;
  * gradients of 3 and 4, normalized FP32 Hessians of 14 and 15), so do the results of
  * one point in calls of different size, as of a set in one call and split over
  * GPUs; name the family to have them equal. sphericart_compute_host chooses by
- * the whole call. Launch shapes and lanes per point do not change results.
+ * the whole call. Tile shapes do not change results, nor do the lanes of DEGREE in
+ * FP64.
  *   POINT:  one thread per point, the whole (l, m) recursion unrolled in
  *           registers for a compile-time l_max, outputs staged in shared memory
  *           and written with bulk (TMA) copies.

@@ -563,15 +563,18 @@ bool point_hybrid_wins(int l_max, int dtype, bool grad) {
 namespace {
 
 // FP64 arithmetic on FP32 storage at small l_max: POINT_HC's one lane per point,
-// whole rows by bulk copies, against DEGREE's stage of a few degrees (400k
-// points, gradients, us: l_max 1 89 on DEGREE, 17 for POINT_HC in FP64; 2 140 /
-// 27; 3 189 / 70; 4 275 / 136; 5 357 / 240, but the conversions of the outputs run
-// on the FP64 pipe in POINT, 144 per point there). Gradients of l_max 3 and 4 at few
-// points: DEGREE's split of a point over lanes (3: 4k points 9.0 / 11.5, 8k 12.1 /
-// 11.7; 4: 11.8 / 17.0, 15.4 / 17.3, 10k 19 / 17.3); values stay on POINT_HC (3, 4k
-// points: 6.0 / 4.7; 4: 7.4 / 6.4).
-bool mixed_prefers_point(int64_t n, int l_max, bool grad) {
-    return l_max <= kMixedHcMaxL && (l_max <= 2 || !grad || n >= 8192);
+// whole rows by bulk copies, against DEGREE's stage of a few degrees (400k points,
+// gradients, scaled / normalized, us, POINT_HC and DEGREE: l_max 1 10, 85 / 54, 138;
+// 2 34, 130 / 111, 190; 3 80, 176 / 208, 236; 4 185, 252 / 359, 324), but the
+// conversions of the outputs run on the FP64 pipe in POINT, 144 per point at l_max 5.
+// Gradients of l_max 3 and 4 at few points: DEGREE's split of a point over lanes
+// (normalized, POINT_HC and DEGREE: 3, 4k points 11.5, 9.0, 8k 11.7, 12.1; 4, 4k 17.0,
+// 11.8, 10k 17.3, 19, 30k 41, 42, 100k 101, 101); values stay on POINT_HC (3, 4k
+// points: 4.7, 6.0; 4: 6.4, 7.4).
+bool mixed_prefers_point(int64_t n, int l_max, bool grad, bool normalized) {
+    if (l_max > kMixedHcMaxL) return false;
+    if (l_max <= 2 || !grad) return true;
+    return n >= 8192 && (l_max < 4 || !normalized || n < 65536);
 }
 
 }  // namespace
@@ -706,7 +709,7 @@ int compute_routed(const void* xyz, int64_t n, int l_max, int normalized, int dt
     }
     int hc = 0;
     const bool mixed_point = kernel == SPH_KERNEL_AUTO && !launch && mixed && !ddsph && out == SPH_OUT_SAME &&
-                             mixed_prefers_point(n_call, l_max, grad);
+                             mixed_prefers_point(n_call, l_max, grad, normalized);
     if (mixed_point) {
         fam = SPH_KERNEL_POINT;
         hc = 1;

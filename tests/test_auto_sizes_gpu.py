@@ -43,6 +43,7 @@ def test_fp64_bounds(l_max, normalized, grad, n, degree):
 
 
 @pytest.mark.parametrize("l_max,grad,n,degree", [(3, True, 8191, True), (4, True, 8192, False), (4, False, 100, False),
+                                                 (4, True, 65_535, False), (4, True, 65_536, True),
                                                  (2, True, 100, False), (5, True, 9000, True)])
 def test_mixed_bounds(l_max, grad, n, degree):
     x = _x(n, torch.float32)
