@@ -485,8 +485,8 @@ int sphericart_tune_clear(void);
  * events on `stream`; synchronises), installs the fastest for later calls
  * with launch == NULL (as sphericart_set_launch) and returns it in *best
  * (and its time in *best_ms if non-NULL). Where AUTO runs this many SPH_F64
- * points on DEGREE, and DEGREE is faster than every shape, none is installed
- * (an installed one is removed) and *best is {0, 0, 0, 0}. l_max <= SPH_MAX_L_POINT, n > 0.
+ * points on DEGREE, and DEGREE is faster than every shape, AUTO stays there and
+ * the shape is that of calls which name POINT. l_max <= SPH_MAX_L_POINT, n > 0.
  * The autotuner and the batch autotuner are the project's own: the paper
  * grows its shared-memory allocation on first call instead (Section 3). */
 int sphericart_autotune(const void* xyz, int64_t n, int l_max, int normalized,
@@ -506,12 +506,13 @@ int sphericart_batch_autotune(const sph_batch_set* sets, int nsets, void* stream
 
 /* sphericart_tune_export: writes the tuned POINT shapes of the current device
  * as text lines "gpu_name l_max dtype out grad P W B lanes" into buf (NUL-terminated,
- * truncated to len); *needed receives the full size. Host memory. */
+ * truncated to len); *needed receives the full size. Host memory. A line ends in
+ * " 0" where AUTO stays on DEGREE (sphericart_autotune). */
 int sphericart_tune_export(char* buf, size_t len, size_t* needed);
 
 /* sphericart_tune_import: installs the lines of `text` whose gpu_name matches
- * the current device (others are skipped; a missing lanes field reads as 0);
- * *imported receives the count. */
+ * the current device (others are skipped; a missing lanes field reads as 0, the
+ * one after it as 1); *imported receives the count. */
 int sphericart_tune_import(const char* text, int* imported);
 
 /* sphericart_fma_peak: measures this device's fused multiply-add throughput

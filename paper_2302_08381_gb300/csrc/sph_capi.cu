@@ -268,7 +268,7 @@ uint32_t* device_status_word() {
 namespace {
 
 using TuneKey = std::tuple<int, int, int, int, int>;  // device, L, dtype, out, grad
-std::map<TuneKey, sph_launch> g_tuned;
+std::map<TuneKey, TunedShape> g_tuned;
 
 int elem_size(int dtype, int out) {
     if (dtype == SPH_F64) return 8;
@@ -481,22 +481,16 @@ bool resolve_point16(sph_launch& s, int L) {
 }  // namespace
 
 sph_launch point_fwd_shape(int L, int grad) {
+    TunedShape t;
     sph_launch s{0, 0, 0, 0};
-    if (!tuned_launch(L, SPH_F32, SPH_OUT_SAME, grad, &s)) s = sph_launch{0, 0, 0, 0};
+    if (tuned_launch(L, SPH_F32, SPH_OUT_SAME, grad, &t)) s = t.shape;
     const sph_launch d = default_point_fwd(L, grad, 4, 0);
     if (s.points_per_tile == 0) s.points_per_tile = d.points_per_tile;
     if (s.warps_per_block == 0) s.warps_per_block = d.warps_per_block;
     return s;
 }
 
-void tuned_remove(int L, int dtype, int out, int grad) {
-    int d = -1;
-    if (cudaGetDevice(&d) != cudaSuccess) return;
-    std::lock_guard<std::mutex> lk(g_mu);
-    g_tuned.erase(TuneKey{d, L, dtype, out, grad});
-}
-
-bool tuned_launch(int L, int dtype, int out, int grad, sph_launch* s) {
+bool tuned_launch(int L, int dtype, int out, int grad, TunedShape* s) {
     int d = -1;
     if (cudaGetDevice(&d) != cudaSuccess) {
         cudaGetLastError();
@@ -668,6 +662,50 @@ int ensure_device(const char* what) {
 
 namespace sph {
 
+int install_shape(int l_max, int dtype, int out, int grad, const sph_launch* launch, bool for_auto) {
+    if (!launch || l_max < 0 || l_max > SPH_MAX_L_POINT || (dtype != SPH_F32 && dtype != SPH_F64) ||
+        (out != SPH_OUT_SAME && out != SPH_OUT_BF16)) {
+        set_error("set_launch: bad arguments");
+        return SPH_EINVAL;
+    }
+    int st = ensure_device("set_launch");
+    if (st) return st;
+    const int eo = elem_size(dtype, out);
+    const int g = grad >= 2 ? 2 : (grad ? 1 : 0);  // 2: values + gradients + Hessians
+    sph_launch s = *launch;
+    if (s.lanes_per_point != 0 && s.lanes_per_point != 1 && s.lanes_per_point != 4 && s.lanes_per_point != 10 &&
+        s.lanes_per_point != 16) {
+        set_error("set_launch: POINT lanes_per_point must be 0, 1, 4, 10 or 16");
+        return SPH_EINVAL;
+    }
+    if (s.lanes_per_point == 10 || s.lanes_per_point == 16) {
+        if (g != 2 || dtype != SPH_F32 || out != SPH_OUT_SAME) {
+            set_error("set_launch: 10 or 16 lanes per point take FP32 arithmetic and storage with Hessians");
+            return SPH_EINVAL;
+        }
+        if (!(s.lanes_per_point == 10 ? resolve_point10(s, l_max) : resolve_point16(s, l_max))) return SPH_EINVAL;
+    } else if (s.lanes_per_point == 4) {
+        if (g != 1 || dtype != SPH_F32) {
+            set_error("set_launch: 4 lanes per point take FP32 arithmetic, values and gradients");
+            return SPH_EINVAL;
+        }
+        if (!resolve_point(s, default_point4_fwd(l_max, eo), l_max, eo, point4_row_bytes(l_max, eo)))
+            return SPH_EINVAL;
+        if (s.points_per_tile > 8) {
+            set_error("set_launch: 4 lanes per point take points_per_tile <= 8");
+            return SPH_EINVAL;
+        }
+    } else if (!resolve_point(s, default_point_fwd(l_max, g ? 1 : 0, eo, g == 2), l_max, eo,
+                              point_row_bytes(l_max, g ? 1 : 0, eo, g == 2))) {
+        return SPH_EINVAL;
+    }
+    int d = -1;
+    cudaGetDevice(&d);
+    std::lock_guard<std::mutex> lk(g_mu);
+    g_tuned[TuneKey{d, l_max, dtype, out, g}] = TunedShape{s, for_auto};
+    return SPH_OK;
+}
+
 int compute_routed(const void* xyz, int64_t n, int l_max, int normalized, int dtype, int out, int qprec, int kernel,
                    const sph_launch* launch, void* sph, void* dsph, void* ddsph, void* stream, int64_t n_call) {
     int st = check_common(n, l_max, dtype, kernel);
@@ -694,9 +732,9 @@ int compute_routed(const void* xyz, int64_t n, int l_max, int normalized, int dt
     const bool hess_bf16 = ddsph && out == SPH_OUT_BF16;
     if (fam == SPH_KERNEL_AUTO)
         fam = auto_family(l_max, dtype, out, qprec, ddsph != nullptr, dsph != nullptr, normalized, n_call);
-    sph_launch installed;
+    TunedShape installed;
     if (kernel == SPH_KERNEL_AUTO && !launch && !ddsph && f64_prefers_degree(n_call, l_max, dtype, grad, normalized) &&
-        !tuned_launch(l_max, dtype, out, grad, &installed)) {  // an installed shape is a POINT shape
+        !(tuned_launch(l_max, dtype, out, grad, &installed) && installed.for_auto)) {
         // POINT needs no device tables: a call captured before any upload stays
         // there, and so does one whose upload fails
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -763,8 +801,8 @@ int compute_routed(const void* xyz, int64_t n, int l_max, int normalized, int dt
             cudaGetDevice(&d);
             std::lock_guard<std::mutex> lk(g_mu);
             auto it = g_tuned.find(TuneKey{d, l_max, dtype, out, ddsph ? 2 : grad});
-            if (it != g_tuned.end() && !(hc && it->second.lanes_per_point == 4)) {
-                a.launch = it->second;
+            if (it != g_tuned.end() && !(hc && it->second.shape.lanes_per_point == 4)) {
+                a.launch = it->second.shape;
                 from_default = false;
             }
         }
@@ -1069,7 +1107,7 @@ int sphericart_launch_info(int l_max, int dtype, int out, int grad, int hess, in
         {
             std::lock_guard<std::mutex> lk(g_mu);
             auto it = g_tuned.find(TuneKey{d, l_max, dtype, out, hess ? 2 : (grad ? 1 : 0)});
-            if (it != g_tuned.end()) s = it->second;
+            if (it != g_tuned.end()) s = it->second.shape;
         }
         const bool none = s.points_per_tile == 0 && s.warps_per_block == 0 && s.blocks_per_sm == 0 &&
                           s.lanes_per_point == 0;
@@ -1096,47 +1134,7 @@ int sphericart_launch_info(int l_max, int dtype, int out, int grad, int hess, in
 }
 
 int sphericart_set_launch(int l_max, int dtype, int out, int grad, const sph_launch* launch) {
-    if (!launch || l_max < 0 || l_max > SPH_MAX_L_POINT || (dtype != SPH_F32 && dtype != SPH_F64) ||
-        (out != SPH_OUT_SAME && out != SPH_OUT_BF16)) {
-        set_error("set_launch: bad arguments");
-        return SPH_EINVAL;
-    }
-    int st = ensure_device("set_launch");
-    if (st) return st;
-    const int eo = elem_size(dtype, out);
-    const int g = grad >= 2 ? 2 : (grad ? 1 : 0);  // 2: values + gradients + Hessians
-    sph_launch s = *launch;
-    if (s.lanes_per_point != 0 && s.lanes_per_point != 1 && s.lanes_per_point != 4 && s.lanes_per_point != 10 &&
-        s.lanes_per_point != 16) {
-        set_error("set_launch: POINT lanes_per_point must be 0, 1, 4, 10 or 16");
-        return SPH_EINVAL;
-    }
-    if (s.lanes_per_point == 10 || s.lanes_per_point == 16) {
-        if (g != 2 || dtype != SPH_F32 || out != SPH_OUT_SAME) {
-            set_error("set_launch: 10 or 16 lanes per point take FP32 arithmetic and storage with Hessians");
-            return SPH_EINVAL;
-        }
-        if (!(s.lanes_per_point == 10 ? resolve_point10(s, l_max) : resolve_point16(s, l_max))) return SPH_EINVAL;
-    } else if (s.lanes_per_point == 4) {
-        if (g != 1 || dtype != SPH_F32) {
-            set_error("set_launch: 4 lanes per point take FP32 arithmetic, values and gradients");
-            return SPH_EINVAL;
-        }
-        if (!resolve_point(s, default_point4_fwd(l_max, eo), l_max, eo, point4_row_bytes(l_max, eo)))
-            return SPH_EINVAL;
-        if (s.points_per_tile > 8) {
-            set_error("set_launch: 4 lanes per point take points_per_tile <= 8");
-            return SPH_EINVAL;
-        }
-    } else if (!resolve_point(s, default_point_fwd(l_max, g ? 1 : 0, eo, g == 2), l_max, eo,
-                              point_row_bytes(l_max, g ? 1 : 0, eo, g == 2))) {
-        return SPH_EINVAL;
-    }
-    int d = -1;
-    cudaGetDevice(&d);
-    std::lock_guard<std::mutex> lk(g_mu);
-    g_tuned[TuneKey{d, l_max, dtype, out, g}] = s;
-    return SPH_OK;
+    return install_shape(l_max, dtype, out, grad, launch, true);
 }
 
 int sphericart_tune_clear(void) {

@@ -196,8 +196,12 @@ BatchOneFn batch_one_fn(int gn);
 
 // Tuned POINT forward shape installed for (l_max, dtype, out, grad) on the
 // current device; false if none.
-bool tuned_launch(int L, int dtype, int out, int grad, sph_launch* s);
-void tuned_remove(int L, int dtype, int out, int grad);
+struct TunedShape {
+    sph_launch shape;
+    bool for_auto;  // AUTO stays on POINT for it where it goes by the number of points
+};
+bool tuned_launch(int L, int dtype, int out, int grad, TunedShape* s);
+int install_shape(int L, int dtype, int out, int grad, const sph_launch* launch, bool for_auto);
 
 // The POINT forward launch shape for FP32 values (+ gradients when grad) at
 // this l_max on the current device: the tuned one if installed, else the

@@ -203,22 +203,18 @@ int sphericart_autotune(const void* xyz, int64_t n, int l_max, int normalized, i
         set_error("autotune: no launchable shape");
         return SPH_EUNSUPPORTED;
     }
+    // with no shape installed AUTO may run DEGREE here: that stays so where it is the faster
+    bool for_auto = true;
     if (f64_prefers_degree(n, l_max, dtype, grad != 0, normalized != 0) &&
         sphericart_compute_ex(xyz, n, l_max, normalized, dtype, out, SPH_Q_NATIVE, SPH_KERNEL_DEGREE, nullptr, sph,
                               dsph, nullptr, stream) == SPH_OK) {
-        // with no shape installed AUTO runs DEGREE here: that stays so where it is the faster
         const float t = median(SPH_KERNEL_DEGREE, nullptr);
         if (t < 0.f) return SPH_ECUDA;
-        if (t <= best_t) {
-            tuned_remove(l_max, dtype, out, grad);
-            *best = sph_launch{0, 0, 0, 0};
-            if (best_ms) *best_ms = t;
-            return SPH_OK;
-        }
+        for_auto = best_t < t;
     }
     *best = best_s;
     if (best_ms) *best_ms = best_t;
-    return sphericart_set_launch(l_max, dtype, out, grad, &best_s);
+    return install_shape(l_max, dtype, out, grad, &best_s, for_auto);
 }
 
 int sphericart_batch_autotune(const sph_batch_set* sets, int nsets, void* stream, int reps, sph_launch* best,
@@ -287,12 +283,12 @@ int sphericart_tune_export(char* buf, size_t len, size_t* needed) {
             for (int out = 0; out <= 1; ++out)
                 for (int grad = 0; grad <= 2; ++grad) {
                     if (dt == SPH_F64 && out == SPH_OUT_BF16) continue;
-                    int fam = 0;
-                    sph_launch s{0, 0, 0, 0};
-                    if (!tuned_launch(L, dt, out, grad, &s)) continue;
-                    (void)fam;
+                    TunedShape t;
+                    if (!tuned_launch(L, dt, out, grad, &t)) continue;
+                    const sph_launch& s = t.shape;
                     os << name << ' ' << L << ' ' << dt << ' ' << out << ' ' << grad << ' ' << s.points_per_tile
-                       << ' ' << s.warps_per_block << ' ' << s.blocks_per_sm << ' ' << s.lanes_per_point << '\n';
+                       << ' ' << s.warps_per_block << ' ' << s.blocks_per_sm << ' ' << s.lanes_per_point
+                       << (t.for_auto ? "" : " 0") << '\n';
                 }
     const std::string text = os.str();
     if (needed) *needed = text.size() + 1;
@@ -321,8 +317,10 @@ int sphericart_tune_import(const char* text, int* imported) {
         if (gpu != name) continue;
         int lanes = 0;  // optional 9th field: lanes_per_point
         if (!(ls >> lanes)) lanes = 0;
+        int for_auto = 1;  // optional 10th field
+        if (!(ls >> for_auto)) for_auto = 1;
         sph_launch s{P, W, B, lanes};
-        if (sphericart_set_launch(L, dt, out, grad, &s) == SPH_OK) ++count;
+        if (install_shape(L, dt, out, grad, &s, for_auto != 0) == SPH_OK) ++count;
     }
     if (imported) *imported = count;
     return SPH_OK;

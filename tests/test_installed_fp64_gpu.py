@@ -1,6 +1,6 @@
 """POINT shapes installed for FP64 requests that AUTO otherwise runs on DEGREE by
-the number of points: AUTO runs them, and the autotuner installs none where
-DEGREE is faster. Which kernel ran is told by its bits."""
+the number of points: AUTO runs them, but not the autotuner's where DEGREE is
+faster. Which kernel ran is told by its bits."""
 
 import pytest
 import torch
@@ -42,12 +42,20 @@ def test_auto_runs_an_installed_shape(l_max, n, grad):
     assert _equal(auto(), degree)
 
 
-def test_autotune_keeps_degree_where_it_is_faster():
+def test_autotune_keeps_degree_where_it_is_faster(tmp_path):
     x = _x(60_000)
+    auto = lambda: api.spherical_harmonics(x, 8, True, gradients=True)  # noqa: E731
+    point, degree = (api.spherical_harmonics(x, 8, True, gradients=True, kernel=k) for k in ("point_hc", "degree"))
     C.sphericart_set_launch(8, C.SPH_F64, C.SPH_OUT_SAME, 1, C.make_launch(16, 1, 4, 0))
     shape, ms = api.autotune(x, 8, True, reps=1)  # DEGREE takes about 0.6 of the time here
-    assert ms > 0 and not any(shape.values())
-    assert _equal(api.spherical_harmonics(x, 8, True, gradients=True),
-                  api.spherical_harmonics(x, 8, True, gradients=True, kernel="degree"))
-    shape, ms = api.autotune(x, 4, True, reps=1)  # (AUTO: POINT)
-    assert ms > 0 and shape["points_per_tile"] > 0
+    assert ms > 0 and _equal(auto(), degree)
+    fam, s = C.sphericart_launch_info(8, C.SPH_F64, C.SPH_OUT_SAME, 1, 0)  # (of calls that name POINT_HC)
+    assert fam == C.SPH_KERNEL_POINT_HC and s.points_per_tile == shape["points_per_tile"] > 0
+    # a saved table keeps that; one without the last field installs for AUTO
+    path = tmp_path / "tune.txt"
+    api.save_tuning(str(path))
+    C.sphericart_tune_clear()
+    assert api.load_tuning(str(path)) == 1 and _equal(auto(), degree)
+    line = path.read_text().split()
+    assert len(line) == 10 and C.sphericart_tune_import(" ".join(line[:9])) == 1
+    assert _equal(auto(), point)
