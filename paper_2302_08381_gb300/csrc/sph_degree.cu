@@ -16,11 +16,11 @@
 //    are read from a per-lane table (m descends) and the gradients of Eq.
 //    iter-deri read the previous degree's column, updated in place.
 //
-// With the upward recursion a point may also be split over LPP = 2 or 4
-// lanes (a warp then owns 32/LPP points): lane h of a point runs the channels
-// m = h (mod LPP) and steps c_m, s_m by (x + i y)^LPP. The per-warp shared
-// memory shrinks by LPP, so more warps are resident to hide the latency of
-// the shared-memory traffic.
+// With the upward recursion a point may also be split over LPP = 2, 4 or (FP64
+// arithmetic) 8 lanes (a warp then owns 32/LPP points): lane h of a point runs the
+// channels m = h (mod LPP); with FP32 arithmetic it steps c_m, s_m by
+// (x + i y)^LPP. The per-warp shared memory shrinks by LPP, so more warps are
+// resident to hide the latency of the shared-memory traffic.
 //
 // Outputs: the columns of one degree are contiguous in every output row
 // (l*l .. l*l+2l). A degree is produced in chunks of up to 16 m values (at
@@ -31,8 +31,8 @@
 // two contiguous row segments.
 //
 // The translation unit is compiled once per variant: SPH_DEGREE_DOWN=1 defines
-// the downward-in-m entry point; SPH_DEGREE_DOWN=0 with SPH_DEGREE_LPP = 1, 2
-// or 4 the upward-in-l entry point for that many lanes per point.
+// the downward-in-m entry point; SPH_DEGREE_DOWN=0 with SPH_DEGREE_LPP = 1, 2,
+// 4 or 8 the upward-in-l entry point for that many lanes per point.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -446,8 +446,8 @@ __global__ void __launch_bounds__(256) degree_fwd_kernel(const TI* __restrict__ 
 //    products (scaled: 6 and 12; values: 2 and 4);
 //  * ten of those products (values: all four) run on the integer pipe, whose
 //    issue slots idle beside the FP64 pipe (sph_mul64.cuh).
-// 200k points, l_max 30, normalized, values and gradients: 9.03 -> 3.92 ms (FP64
-// pipe about 60 % busy, issue 50 %). Linear maps from the columns of degree l - 1
+// 200k points, l_max 30, normalized, values and gradients: 9.03 -> 3.75 ms (FP64
+// pipe 71 % busy, issue 54 %). Linear maps from the columns of degree l - 1
 // take one FP64 instruction less, and were 2 % faster, but carry the larger
 // rounding of the m = 0 column into the gradients next to the poles (rms error
 // 7.9e-15 against 4.5e-15): not kept.
@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(GRAD ? 256 : 320, 2) degree_f64_kernel(const T
         // A point with a zero coordinate has a zero Qtilde, c_m or s_m at every
         // second step, and trying those steps on the integer pipe first cost more than
         // it gains (200k points with z = 0, us, with the trial / now: values, l_max 12
-        // 354 / 239, 20 885 / 600; gradients, l_max 8 659 / 537, 20 3063 / 2433). Values
+        // 354 / 243, 20 885 / 616; gradients, l_max 8 660 / 527, 20 3067 / 2382). Values
         // take a copy of the loop whose products accept zeros. With gradients that is
         // too much code; those tiles run on the FP64 pipe alone, scaled in a copy of
         // the loop (a flag in the one loop: random points 1..5 % slower), normalized

@@ -24,9 +24,11 @@ constexpr int kExpansionMaxRad = 64;
 // Row layout of the staged harmonics: the 2l+1 columns of degree l in groups
 // of 4 slots (the last group of a degree padded with zeros), group g at word
 // 4g, so that a lane stores and loads a group with one 16-byte access (FP32).
-// The contraction is bound by instruction issue and shared-memory wavefronts
-// (64 % and 74 % busy): one load per point and lane instead of four, and 16
-// stores of a group per point instead of one per column.
+// One load per point and lane instead of four, and 16 stores of a group per point
+// instead of one per column (100k centres, l_max 6, 8 radial: 0.267 -> 0.245 ms). With
+// a load and a store per column the kernel was at the limit of issue and of
+// shared-memory wavefronts (64 % and 74 % busy); now it is latency at 11 warps per SM
+// (issue 48 %, wait 1.8 of the stall cycles per instruction).
 __host__ __device__ constexpr int exp_gstart(int l) { return l == 0 ? 0 : l + (l - 1) * (l - 1) / 4; }
 // Row stride in words: 4 times an odd number, so that the 8 lanes of a quarter
 // warp, each storing a group of its own row, cover all 32 banks.
@@ -110,8 +112,8 @@ constexpr int kExpBatch = 32;  // centres whose CSR offsets a warp holds in regi
 // contraction while the next chunk's rows were prefetched into L2, leaves
 // room for 12 resident warps per SM where two buffers (the next chunk's rows
 // loaded into shared memory during the current one) leave 8: measured on
-// GB300, 0.267 against 0.369 ms (l_max 6, 8 radial, 100k centres x ~40
-// points).
+// GB300 before the grouped accesses above, 0.267 against 0.369 ms (l_max 6, 8
+// radial, 100k centres x ~40 points).
 constexpr int kExpRBuf = 1;
 
 // Per-warp shared memory: Y rows of a 32-point chunk (grouped layout),
