@@ -622,8 +622,8 @@ int row_shape(const void* kern, int64_t n, int cap, size_t per_warp, size_t tabl
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(r->smem));
         if (e != cudaSuccess) return int(e);
     }
-    int64_t bps = asked > 0 ? std::max<int64_t>(1, asked / r->W) : s.blocks_per_sm;
-    if (bps <= 0) {
+    int64_t bps = asked > 0 ? std::max<int64_t>(1, asked / r->W) : 0;
+    if (bps == 0) {
         int occ = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * r->W, r->smem) != cudaSuccess) {
             cudaGetLastError();
