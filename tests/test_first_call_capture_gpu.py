@@ -1,6 +1,6 @@
 """First FP64 calls of a process around a graph capture. The tables they need are
 uploaded without disturbing a capture that another stream has going on; under
-capture themselves they run on kernels that need none."""
+capture themselves they run on kernels that need none, where there is one."""
 
 import os
 import subprocess
@@ -54,8 +54,22 @@ torch.cuda.synchronize()
 assert same(out, degree)
 """
 
+# a kernel that needs tables, first called under capture: they are uploaded at once
+NEEDED = """
+z = torch.randn(70_000, 3, device="cuda")
+mixed = lambda o, **kw: api.spherical_harmonics(z, 4, True, gradients=True, qprec="f64", out=o, **kw)
+a, b = ((torch.empty(70_000, 25, device="cuda"), torch.empty(70_000, 3, 25, device="cuda")) for _ in range(2))
+torch.cuda.synchronize()
+with torch.cuda.graph(graph):
+    mixed(a)
+graph.replay()
+torch.cuda.synchronize()
+mixed(b, kernel="degree")
+assert same(a, b)
+"""
 
-@pytest.mark.parametrize("body", [ELSEWHERE, ITSELF], ids=["elsewhere", "itself"])
+
+@pytest.mark.parametrize("body", [ELSEWHERE, ITSELF, NEEDED], ids=["elsewhere", "itself", "needed"])
 def test_first_fp64_call(body):
     r = subprocess.run([sys.executable, "-c", SETUP + body], capture_output=True, text=True, cwd=ROOT, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
